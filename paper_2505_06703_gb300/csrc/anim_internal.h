@@ -290,8 +290,10 @@ struct RasterArgs {
   uint32_t *rgba;                 // nullable
   int width, height, cols;
   float spacing, ox, oy, scale;
+  int stage_verts;                // set by launch_raster: vertices the shared-memory stage holds
 };
-cudaError_t launch_raster(const RasterArgs &a, int n_chars, cudaStream_t s);
+// max_verts: the largest vertex count among the characters' types.
+cudaError_t launch_raster(const RasterArgs &a, int n_chars, int max_verts, cudaStream_t s);
 
 // Setup kernels.
 cudaError_t launch_prepare_keys(float4 *keys, int n_clips, int n_keys, int n, cudaStream_t s);

@@ -1392,7 +1392,9 @@ int anim_raster(anim_ctx *ctx, const anim_plan *plan, const float *d_verts, cons
   a.ox = params->ox;
   a.oy = params->oy;
   a.scale = params->scale;
-  CK(launch_raster(a, (int)plan->n_chars, (cudaStream_t)stream));
+  int max_verts = 0;
+  for (int t : plan->used) max_verts = std::max(max_verts, ctx->types[t]->n_verts);
+  CK(launch_raster(a, (int)plan->n_chars, max_verts, (cudaStream_t)stream));
   return ANIM_OK;
 }
 
