@@ -47,9 +47,10 @@ struct TypeDev {
   // The paper's 64-node blocks (comparator kernels): nearest ancestor of
   // each joint outside its block of 64 consecutive indices, -1 at the top.
   const int32_t *blk_out;
-  // Skinned mesh (linear blend skinning after the bind product): 3 float4
-  // per vertex: (px py pz nx), (ny nz w0 w1), (w2 w3 bones01 bones23) with
-  // the bone ids as 16-bit pairs in the last two words' bits.
+  // Skinned mesh (linear blend skinning after the bind product): 3 planes of
+  // n_verts float4, (px py pz nx), (ny nz w0 w1), (w2 w3 bones01 bones23)
+  // with the bone ids as 16-bit pairs in the last two words' bits; planes, so
+  // that a warp's loads are contiguous.
   int n_verts;
   int n_faces;
   const float4 *mesh;
@@ -119,7 +120,7 @@ struct LaunchCfg {
 };
 
 // ---------------------------------------------------------------- kernels
-// Arguments of the persistent scan kernels (k_scan_qt's modes, k_scan).
+// Arguments of the persistent scan kernel (k_scan_qt's modes).
 struct ScanArgs {
   const TypeDev *types;
   const WorkItem *items;
@@ -148,9 +149,6 @@ struct ScanArgs {
   const float *layer_w;
   const float *add_w;
 };
-
-// The matrix frame kernel with the skinning pass (a.verts).
-cudaError_t launch_scan(const ScanArgs &a, const LaunchCfg &cfg, cudaStream_t s);
 
 // Frame work queue.  The plan cuts the characters of each type (types in
 // cost order) into ranges of at most kRangeChars (kRangeCharsMax for the
@@ -300,14 +298,19 @@ cudaError_t launch_prepare_keys(float4 *keys, int n_clips, int n_keys, int n, cu
 cudaError_t launch_bind_from_rest(const int32_t *parent, const float *rest_q, const float *rest_t, int n,
                                   float4 *inv_bind, cudaStream_t s);
 
-// Shared-memory footprint of one work item of C characters (bytes).
+// Shared-memory footprint of one work item of C characters (bytes): as 3x4
+// matrices (the form that decides which types a plan takes, and that the
+// allocation-free entry runs on), the adjoint's, (q, t) pairs, and (q, t)
+// pairs with the third plane of the frame with skinning.
 size_t scan_smem_bytes(int n, int nseg, int C);
 size_t adjoint_smem_bytes(int n, int nseg, int C);
 size_t scan_qt_smem_bytes(int n, int nseg, int C);
+size_t scan_skin_smem_bytes(int n, int nseg, int C);
 
 // The scan on (quaternion, translation) items: mode 0 the plain frame (skin
 // matrices out), mode 1 the forward from local poses (skin and / or model
-// matrices out), mode 2 the frame with layered blending.
+// matrices out), mode 2 the frame with layered blending, mode 3 the plain
+// frame with the skinning pass (a.verts).
 cudaError_t launch_scan_qt(int mode, const ScanArgs &a, const LaunchCfg &cfg, cudaStream_t s);
 
 }  // namespace anim

@@ -428,7 +428,7 @@ struct TypeHost {
   WalkSched ws;                 // chain-walk schedule (mode 0: not walkable)
   bool ws_done = false;
   float4 *d_add = nullptr;      // additive layer keys [n_keys][n][2]
-  float4 *d_mesh = nullptr;     // skinned mesh, 3 float4 per vertex
+  float4 *d_mesh = nullptr;     // skinned mesh, 3 planes of n_verts float4
   int n_verts = 0;
   int32_t *d_faces = nullptr;   // [n_faces][3]
   int n_faces = 0;
@@ -788,7 +788,7 @@ struct anim_plan {
   std::vector<int64_t> row_off;
   std::vector<int> used;                      // type ids, most costly first
   std::vector<std::vector<int32_t>> by_type;  // characters of each used type (indexed like used)
-  std::vector<int> C_scan, C_adj;             // per ctx type id
+  std::vector<int> C_skin, C_adj;             // per ctx type id
   std::vector<int> C_frame;                   // plain frame: characters per (q, t) item
   int64_t total = 0;
   int version = -1;  // schedule version the items were built for
@@ -808,7 +808,7 @@ struct anim_plan {
   int32_t *d_used = nullptr, *d_cap = nullptr;
   LaunchCfg cfg_scan{}, cfg_adj{};
   size_t smem_frame = 0;     // plain frame, (q, t) items
-  size_t smem_frame_mat = 0; // frame with skinning or layers, matrix items
+  size_t smem_skin = 0;      // frame with skinning
   int adj_unfit = -1;
   // frame: item slots [0, n_slots_walk) belong to the chain-walk kernel
   // (queue counters d_queue[0..1]), the rest to the segmented CTA kernel
@@ -967,14 +967,16 @@ size_t adj_budget(const anim_ctx *ctx) {
 }
 
 // Characters per work item: kind 0 the matrix scan, 1 the adjoint, 2 the
-// plain frame's (q, t) items.
+// plain frame's (q, t) items, 3 the frame with skinning's.
 int choose_C(const anim_ctx *ctx, const TypeHost &T, int kind) {
   const bool adjoint = kind == 1;
   const size_t budget = adjoint ? adj_budget(ctx) : smem_budget(ctx);
   int C = std::max(1, std::min(kCMax, ctx->joints_per_item / std::max(1, T.n)));
   auto bytes = [&](int c) {
-    return kind == 1 ? adjoint_smem_bytes(T.n, T.seg.nseg, c)
-                     : kind == 2 ? scan_qt_smem_bytes(T.n, T.seg.nseg, c) : scan_smem_bytes(T.n, T.seg.nseg, c);
+    return kind == 1   ? adjoint_smem_bytes(T.n, T.seg.nseg, c)
+           : kind == 2 ? scan_qt_smem_bytes(T.n, T.seg.nseg, c)
+           : kind == 3 ? scan_skin_smem_bytes(T.n, T.seg.nseg, c)
+                       : scan_smem_bytes(T.n, T.seg.nseg, c);
   };
   while (C > 1 && bytes(C) > budget) --C;
   if (bytes(C) > ctx->smem_optin - kStaticSmemAllowance) return 0;
@@ -1014,7 +1016,7 @@ std::vector<WorkItem> make_items(const anim_plan *P, const std::vector<int> &Cv)
 int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   if (P->version == ctx->version) return ANIM_OK;
   const int nt = (int)ctx->types.size();
-  P->C_scan.assign(nt, 1);
+  P->C_skin.assign(nt, 1);
   P->C_adj.assign(nt, 1);
   P->C_frame.assign(nt, 1);
   P->adj_unfit = -1;
@@ -1026,9 +1028,9 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
       return fail(ctx, ANIM_EUNSUPPORTED,
                   "type %d (%d joints, %d segments) does not fit in shared memory with one character", t, T.n,
                   T.seg.nseg);
-    P->C_scan[t] = cs;
     P->C_frame[t] = std::max(cs, choose_C(ctx, T, 2));  // (q, t) items are smaller
-    smem_s = std::max(smem_s, scan_smem_bytes(T.n, T.seg.nseg, cs));
+    P->C_skin[t] = std::max(cs, choose_C(ctx, T, 3));
+    smem_s = std::max(smem_s, scan_skin_smem_bytes(T.n, T.seg.nseg, P->C_skin[t]));
     smem_q = std::max(smem_q, scan_qt_smem_bytes(T.n, T.seg.nseg, P->C_frame[t]));
     // the adjoint keeps two more vectors per joint: a schedule may fit the
     // forward kernels and not the adjoint, which then refuses to run
@@ -1098,8 +1100,8 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   P->n_ranges = (int)ranges.size();
   P->n_slots = slots;
   CK(upload_vec(&P->d_ranges, ranges));
-  // layouts of every type on one kernel: matrix items (the frame with
-  // skinning) and (q, t) items (the frame with layered blending)
+  // layouts of every type on one kernel: the frame with skinning's items and
+  // the frame with layered blending's
   auto all_types = [&](const std::vector<int> &Cv, std::vector<RangeDev> &out) {
     int sl = 0;
     for (size_t u = 0; u < P->used.size(); ++u) {
@@ -1118,11 +1120,11 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
     return sl;
   };
   std::vector<RangeDev> ranges_cta, ranges_qa;
-  const int slots_cta = all_types(P->C_scan, ranges_cta), slots_qa = all_types(P->C_frame, ranges_qa);
+  const int slots_cta = all_types(P->C_skin, ranges_cta), slots_qa = all_types(P->C_frame, ranges_qa);
   P->n_ranges_cta = (int)ranges_cta.size();
   P->n_slots_cta = slots_cta;
   CK(upload_vec(&P->d_ranges_cta, ranges_cta));
-  CK(upload_vec(&P->d_cap_cta, P->C_scan));
+  CK(upload_vec(&P->d_cap_cta, P->C_skin));
   P->n_ranges_qa = (int)ranges_qa.size();
   P->n_slots_qa = slots_qa;
   CK(upload_vec(&P->d_ranges_qa, ranges_qa));
@@ -1143,7 +1145,7 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
     P->cfg_adj = {kAdjThreads, std::max(1, std::min(grid, P->n_items_adj)), std::max<size_t>(smem_a, 16),
                   ctx->ctas_per_sm >= 3 ? 3 : 2};
   P->smem_frame = std::max<size_t>(smem_f, 16);
-  P->smem_frame_mat = std::max<size_t>(smem_s, 16);
+  P->smem_skin = std::max<size_t>(smem_s, 16);
   P->version = ctx->version;
   return ANIM_OK;
 }
@@ -1318,15 +1320,33 @@ int anim_upload_mesh(anim_ctx *ctx, int32_t type_id, int n_verts, const float *r
       if (b < 0 || b >= T.n) return fail(ctx, ANIM_EINVAL, "vertex %d: bone %d out of range", v, b);
       if (!std::isfinite(w)) return fail(ctx, ANIM_EINVAL, "vertex %d: non-finite weight", v);
     }
-    const float *p = rest_pos + 3 * v, *q = rest_nrm + 3 * v, *w = weights + 4 * v;
-    const int32_t *b = bones + 4 * v;
+    const float *p = rest_pos + 3 * v, *q = rest_nrm + 3 * v;
+    // Zero-weight slots are skipped: each takes half of the weight, and the
+    // bone, of the slot that has the most, so that the kernel need not test
+    // (a branch per slot cost it 5 of 113 us) and no unused bone's pose, be
+    // it non-finite, enters the sum.
+    float w[4];
+    int32_t b[4];
+    for (int k = 0; k < 4; ++k) {
+      w[k] = weights[4 * v + k];
+      b[k] = bones[4 * v + k];
+    }
+    for (int k = 0; k < 4; ++k) {
+      if (w[k] != 0.f) continue;
+      int m = 0;
+      for (int i = 1; i < 4; ++i)
+        if (std::fabs(w[i]) > std::fabs(w[m])) m = i;
+      w[m] *= 0.5f;
+      w[k] = w[m];
+      b[k] = b[m];
+    }
     const uint32_t b01 = (uint32_t)b[0] | ((uint32_t)b[1] << 16), b23 = (uint32_t)b[2] | ((uint32_t)b[3] << 16);
     float f01, f23;
     memcpy(&f01, &b01, 4);
     memcpy(&f23, &b23, 4);
-    rec[3 * v] = make_float4(p[0], p[1], p[2], q[0]);
-    rec[3 * v + 1] = make_float4(q[1], q[2], w[0], w[1]);
-    rec[3 * v + 2] = make_float4(w[2], w[3], f01, f23);
+    rec[v] = make_float4(p[0], p[1], p[2], q[0]);
+    rec[(size_t)n_verts + v] = make_float4(q[1], q[2], w[0], w[1]);
+    rec[2 * (size_t)n_verts + v] = make_float4(w[2], w[3], f01, f23);
   }
   CK(cudaSetDevice(ctx->device));
   if (T.d_mesh) cudaFree(T.d_mesh);
@@ -1712,7 +1732,7 @@ int anim_evaluate_frame_skinned(anim_ctx *ctx, const anim_plan *plan, const floa
   if (!d_blend_w || !d_verts) return fail(ctx, ANIM_EINVAL, "NULL device pointer");
   if (!aligned16(d_verts) || (d_skin && !aligned16(d_skin)) || !aligned4(d_blend_w))
     return fail(ctx, ANIM_EINVAL, "d_verts, d_skin must be 16-byte aligned, d_blend_w 4-byte aligned");
-  BucketArgs bk{};  // matrix items of every type
+  BucketArgs bk{};  // items of every type
   bk.ranges = plan->d_ranges_cta;
   bk.n_ranges = plan->n_ranges_cta;
   bk.n_slots = plan->n_slots_cta;
@@ -1740,9 +1760,9 @@ int anim_evaluate_frame_skinned(anim_ctx *ctx, const anim_plan *plan, const floa
   a.verts = d_verts;
   a.vert_off = plan->d_vert_off;
   LaunchCfg cfg = plan->cfg_scan;
-  cfg.ctas = ctx->sm_count * ctx->ctas_per_sm;
-  cfg.smem = plan->smem_frame_mat;
-  CK(launch_scan(a, cfg, (cudaStream_t)stream));
+  cfg.ctas = std::max(1, std::min(ctx->sm_count * ctx->ctas_per_sm, a.n_items));
+  cfg.smem = plan->smem_skin;
+  CK(launch_scan_qt(3, a, cfg, (cudaStream_t)stream));
   return ANIM_OK;
 }
 

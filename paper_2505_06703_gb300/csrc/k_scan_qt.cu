@@ -6,7 +6,11 @@
 //   MODE 1  the forward from given local poses q [total][4] (normalized
 //           here), t [total][3], skin and / or model matrices out;
 //   MODE 2  the frame with layered blending (up to 4 clips by per-character
-//           weights and an additive layer, sample_layers_at).
+//           weights and an additive layer, sample_layers_at);
+//   MODE 3  the plain frame followed by linear blend skinning: the bind pass
+//           leaves the skin matrices' rows in shared memory (a third plane
+//           beside q and t) for the skinning pass, and writes them to global
+//           memory only if the caller wants them.
 // The smaller item footprint lets more characters be in flight per SM, which
 // is what bounds the latency-limited scan passes.  The segment tables are
 // staged by cp.async during pass 1a; one character of a pure chain longer
@@ -14,9 +18,8 @@
 // the segment walks and pointer jumping.  The bind pass normalizes
 // the composed quaternion once (removing the norm drift of long products),
 // forms M = [R(q) | t] and writes M and / or S = M B straight to global
-// memory.  Same item pipeline as k_scan (producer warp, 8 compute warps,
-// work queue); the frame with skinning keeps the matrix form there, as its
-// skinning pass reads the skin matrices from shared memory.
+// memory.  Item pipeline of scan_core.cuh: producer warp, 8 compute warps,
+// work queue.
 #include <cuda_runtime.h>
 
 #include "anim_internal.h"
@@ -79,11 +82,55 @@ __device__ __forceinline__ void chain_scan_qt(int n, float4 *P, QT *wtot, int ti
   compute_sync();
 }
 
+// Linear blend skinning of the item's characters: vertex v of character c
+// goes to sum_k w_k S_{b_k} [p; 1] with normal normalize(sum_k w_k R_{b_k} n)
+// (rigid skin matrices), written as 6 floats at the character's vertex
+// offset.  S is kept in three planes of n rows, character c's from P + c * cs.
+// A thread loads a vertex's record once for the item's characters.
+// Bound by shared-memory bandwidth: a warp reads 4 bones x 3 rows, 48 wave
+// fronts per 32 vertices, 29 of the about 48 us this pass takes of the 104 us
+// frame (4,097 characters, 1,500 vertices each, 147 MB out; 125 us with the
+// scan on 3x4 matrices, 55 without this pass).  Storing through a staging
+// buffer as consecutive words took 3 us more than these 24-byte rows, the
+// streaming hint 1.5 us less.
+__device__ __forceinline__ void skin_mesh(const ItemBuf &b, const float4 *P, int cs, float *verts, int tid) {
+  const int nv = b.T.n_verts, n = b.T.n, C = b.C;
+  const float4 *mesh = b.T.mesh;
+  for (int v = tid; v < nv; v += kComputeThreads) {
+    const float4 r0 = __ldg(mesh + v), r1 = __ldg(mesh + nv + v), r2 = __ldg(mesh + 2 * nv + v);
+    const float w[4] = {r1.z, r1.w, r2.x, r2.y};
+    const uint32_t b01 = __float_as_uint(r2.z), b23 = __float_as_uint(r2.w);
+    for (int c = 0; c < C; ++c) {
+      const float4 *Sc = P + c * cs;
+      float px = 0.f, py = 0.f, pz = 0.f, nx = 0.f, ny = 0.f, nz = 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t bb = k < 2 ? b01 : b23;
+        const float4 *S = Sc + (k & 1 ? bb >> 16 : bb & 0xFFFFu);
+        const float4 s0 = S[0], s1 = S[n], s2 = S[2 * n];
+        px = fmaf(w[k], fmaf(s0.x, r0.x, fmaf(s0.y, r0.y, fmaf(s0.z, r0.z, s0.w))), px);
+        py = fmaf(w[k], fmaf(s1.x, r0.x, fmaf(s1.y, r0.y, fmaf(s1.z, r0.z, s1.w))), py);
+        pz = fmaf(w[k], fmaf(s2.x, r0.x, fmaf(s2.y, r0.y, fmaf(s2.z, r0.z, s2.w))), pz);
+        nx = fmaf(w[k], fmaf(s0.x, r0.w, fmaf(s0.y, r1.x, s0.z * r1.y)), nx);
+        ny = fmaf(w[k], fmaf(s1.x, r0.w, fmaf(s1.y, r1.x, s1.z * r1.y)), ny);
+        nz = fmaf(w[k], fmaf(s2.x, r0.w, fmaf(s2.y, r1.x, s2.z * r1.y)), nz);
+      }
+      const float l2 = nx * nx + ny * ny + nz * nz;
+      const float inv = l2 > 0.f ? rsqrtf(l2) : 0.f;
+      float2 *out = reinterpret_cast<float2 *>(verts + b.voff[c] * 6) + 3 * (size_t)v;
+      __stcs(out + 0, make_float2(px, py));
+      __stcs(out + 1, make_float2(pz, nx * inv));
+      __stcs(out + 2, make_float2(ny * inv, nz * inv));
+    }
+  }
+}
+
 template <int MODE, int MINB>
 __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a) {
   extern __shared__ __align__(128) float4 sm[];
   __shared__ ItemBuf bufs[2];
   __shared__ QT wtot[kComputeWarps];  // chain scan: the warps' run products
+  constexpr int kPlanes = MODE == 3 ? 3 : 2;
   const int tid = threadIdx.x;
   // launched with programmatic stream serialization (after the work-queue
   // kernel, for the frame): wait for the preceding grid to complete before
@@ -105,7 +152,7 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
 
   if (tid >= kComputeThreads) {
     producer_loop<MODE == 1 ? 1 : 0>(bufs, a.queue_head, n_items, a.items, a.types, a.item_chars, a.row_off,
-                                     a.time, a.blend_w, a.status, nullptr,
+                                     a.time, a.blend_w, a.status, MODE == 3 ? a.vert_off : nullptr,
                                      MODE == 2 ? LayerIn{a.layer_w, a.add_w} : LayerIn{nullptr, nullptr}, pf);
     return;
   }
@@ -116,8 +163,9 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
     const ItemBuf &b = bufs[cur];
     if (b.item < 0) break;
     const int C = b.C, n = b.T.n, nseg = b.T.nseg;
-    const int cs2 = 2 * n + 1;  // float4 stride between characters (16 B skew)
-    const ItemLayout Lt = item_layout_qt(sm, C, n, nseg);
+    const int cs2 = 2 * n + 1;  // float4 stride between characters (16 B skew) of pairs
+    const int cs = MODE == 3 ? cs2 + n : cs2;  // with the third plane
+    const ItemLayout Lt = item_layout_qt(sm, C, n, nseg, kPlanes);
     float4 *P = Lt.P;
 
     // ---- pass 1a: local poses (q, t) from the clips or the caller's rows;
@@ -134,14 +182,14 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
         const long long row = b.off[c] + (gat ? __ldg(gat + j) : j);
         const float4 q = normalize4(__ldg(q4 + row));
         const float *tp = a.t + 3 * row;
-        sts_qt(P + c * cs2, j, n, QT{q, make_float4(__ldg(tp), __ldg(tp + 1), __ldg(tp + 2), 0.f)});
+        sts_qt(P + c * cs, j, n, QT{q, make_float4(__ldg(tp), __ldg(tp + 1), __ldg(tp + 2), 0.f)});
       }
     } else if (MODE == 2) {
       // character-minor: the lanes of one joint share its key records
       const int CN = C * n;
       for (int idx = tid; idx < CN; idx += kComputeThreads) {
         const int j = (int)b.divC.div(idx), c = idx - j * C;
-        sts_qt(P + c * cs2, j, n, sample_layers_at(b, j, c));
+        sts_qt(P + c * cs, j, n, sample_layers_at(b, j, c));
       }
     } else {
       const int nk = b.T.n_keys, k0 = b.k0, k1 = (k0 + 1 == nk) ? 0 : k0 + 1;
@@ -178,7 +226,7 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
             ty = fmaf(w, fmaf(al, tb1.y - tb0.y, tb0.y) - ty, ty);
             tz = fmaf(w, fmaf(al, tb1.z - tb0.z, tb0.z) - tz, tz);
           }
-          sts_qt(P + c * cs2, j, n, QT{q, make_float4(tx, ty, tz, 0.f)});
+          sts_qt(P + c * cs, j, n, QT{q, make_float4(tx, ty, tz, 0.f)});
         }
       }
     }
@@ -195,9 +243,9 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
     if (chain) {
       chain_scan_qt(n, P, wtot, tid);
     } else {
-      pass1b_qt(b, Lt, P, cs2, tid);
+      pass1b_qt(b, Lt, P, cs, tid);
       compute_sync();
-      Y = pass2_qt(b, Lt, P, cs2, tid);
+      Y = pass2_qt(b, Lt, P, cs, tid);
     }
 
     // ---- pass 3: model pose, normalize, matrix, (bind,) store
@@ -214,13 +262,26 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
         if (skin) B = ldg_aff(b.T.inv_bind + 3 * j);
         const int c1 = min(C, (grp + 1) * cpt);
         for (int c = grp * cpt; c < c1; ++c) {
-          QT m = lds_qt(P + c * cs2, j, n);
+          QT m = lds_qt(P + c * cs, j, n);
           if (!chain && (info & kJ16Link)) m = qt_mul(lds_qt(Y, c * nseg + g, C * nseg), m);
           const Aff M = aff_from_qt(normalize4(m.q), m.t.x, m.t.y, m.t.z);
           if (model) stg_aff(model4 + (b.off[c] + j) * 3, M);
-          if (skin) stg_aff(skin4 + (b.off[c] + j) * 3, aff_mul(M, B));
+          if (MODE == 3) {  // the joint's own slots: nobody else reads them in this pass
+            const Aff S = aff_mul(M, B);
+            float4 *Pj = P + c * cs + j;
+            Pj[0] = S.r0;
+            Pj[n] = S.r1;
+            Pj[2 * n] = S.r2;
+            if (skin4) stg_aff(skin4 + (b.off[c] + j) * 3, S);
+          } else if (skin) {
+            stg_aff(skin4 + (b.off[c] + j) * 3, aff_mul(M, B));
+          }
         }
       }
+    }
+    if (MODE == 3) {
+      compute_sync();
+      skin_mesh(b, P, cs, a.verts, tid);
     }
     cur ^= 1;
     handoff_sync();
@@ -250,13 +311,16 @@ static cudaError_t launch_qt(const ScanArgs &a, const LaunchCfg &cfg, cudaStream
 
 }  // namespace
 
+size_t scan_smem_bytes(int n, int nseg, int C) { return scan_item_bytes(n, nseg, C); }
 size_t scan_qt_smem_bytes(int n, int nseg, int C) { return qt_item_bytes(n, nseg, C); }
+size_t scan_skin_smem_bytes(int n, int nseg, int C) { return qt_item_bytes(n, nseg, C, 3); }
 
 cudaError_t launch_scan_qt(int mode, const ScanArgs &a, const LaunchCfg &cfg, cudaStream_t st) {
   const bool m3 = cfg.min_blocks >= 3;
   if (mode == 0) return m3 ? launch_qt<0, 3>(a, cfg, st) : launch_qt<0, 2>(a, cfg, st);
   if (mode == 1) return m3 ? launch_qt<1, 3>(a, cfg, st) : launch_qt<1, 2>(a, cfg, st);
-  return m3 ? launch_qt<2, 3>(a, cfg, st) : launch_qt<2, 2>(a, cfg, st);
+  if (mode == 2) return m3 ? launch_qt<2, 3>(a, cfg, st) : launch_qt<2, 2>(a, cfg, st);
+  return m3 ? launch_qt<3, 3>(a, cfg, st) : launch_qt<3, 2>(a, cfg, st);
 }
 
 }  // namespace anim

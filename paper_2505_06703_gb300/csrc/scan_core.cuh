@@ -456,13 +456,14 @@ __device__ __forceinline__ QT qt_identity() {
   return QT{make_float4(0.f, 0.f, 0.f, 1.f), make_float4(0.f, 0.f, 0.f, 0.f)};
 }
 
-// Item layout: P [C][2n + 1] float4 (per character a q plane of n, a t plane
-// of n, one pad), Y0 / Y1 [2][C * nseg] float4 (q plane, t plane), then the
-// type's segment tables as in the matrix layout.
-__device__ __forceinline__ ItemLayout item_layout_qt(float4 *sm, int C, int n, int nseg) {
+// Item layout: P [C][planes n + 1] float4 (per character a q plane of n, a t
+// plane of n -- for the frame with skinning a third, so that its three rows
+// can take the pair's place -- and one pad), Y0 / Y1 [2][C * nseg] float4 (q
+// plane, t plane), then the type's segment tables as in the matrix layout.
+__device__ __forceinline__ ItemLayout item_layout_qt(float4 *sm, int C, int n, int nseg, int planes = 2) {
   ItemLayout L;
   L.P = sm;
-  L.Y0 = L.P + C * (2 * n + 1);
+  L.Y0 = L.P + C * (planes * n + 1);
   L.Y1 = L.Y0 + 2 * C * nseg;
   char *t = reinterpret_cast<char *>(L.Y1 + 2 * C * nseg);
   L.ptr0 = reinterpret_cast<int16_t *>(t);
@@ -530,8 +531,8 @@ __device__ __forceinline__ QT sample_layers_at(const ItemBuf &b, int j, int c) {
   return QT{q, make_float4(tx, ty, tz, 0.f)};
 }
 
-__host__ __device__ inline size_t qt_item_bytes(int n, int nseg, int C) {
-  return 16ull * ((size_t)C * (2 * (size_t)n + 1) + 4ull * C * nseg) + item_table_bytes(n, nseg);
+__host__ __device__ inline size_t qt_item_bytes(int n, int nseg, int C, int planes = 2) {
+  return 16ull * ((size_t)C * (planes * (size_t)n + 1) + 4ull * C * nseg) + item_table_bytes(n, nseg);
 }
 
 // Pass 1b on (q, t) pairs: running products along each segment, in place
