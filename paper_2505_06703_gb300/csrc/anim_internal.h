@@ -11,6 +11,7 @@ namespace anim {
 // "segments": maximal runs of consecutive joints i, i+1, ... with
 // parent[i+1] == i (natural chains), cut into pieces of at most seg_len
 // joints.  Segments partition [0, n) into intervals.
+constexpr int kMaxJumps = 10;  // 2^r < links <= 2,047
 struct TypeDev {
   int n;           // joints
   int nseg;        // segments
@@ -27,10 +28,23 @@ struct TypeDev {
   const uint32_t *jinfo;     // [n] segment of the joint (bits 0-15) | kJStart | kJLink
   // The same tables in the 16-bit form the kernels keep in shared memory,
   // staged there by cp.async: jinfo16 [n rounded up to even] = segment |
-  // kJ16Start | kJ16Link; sub16, par16, gat16 [n] = sub_end, parent and
+  // kJ16Odd | kJ16Start | kJ16Link; sub16, par16, gat16 [n] = sub_end, parent and
   // gather (identity for a type) as int16.
   const uint16_t *jinfo16;
   const int16_t *sub16, *par16, *gat16;
+  // Prefix over the segment tree (pass2_qt).  A segment's links are the parent
+  // joints met on the way to its root: its own seg_link, that of the segment
+  // this lies in, and so on.  hang [n_hang]: the segments with a link, x =
+  // segment | seg_link << 16, y = the second link or ~0.  Then, for r = 1, 2,
+  // ..., the jump_n[r - 1] segments with more than 2^r links, the lists one after
+  // the other in jump, each in index order (mostly consecutive slots, so few
+  // bank conflicts):
+  // segment | the segment 2^r links up << 12 | (that one's value lies in the
+  // odd buffer after r - 1 jumps) << 24.
+  const uint2 *hang;
+  const uint32_t *jump;
+  int n_hang, n_jumps;
+  uint16_t jump_n[kMaxJumps];
   const float4 *inv_bind;    // [n][3] rows of B_i
   const float4 *keys;        // [n_clips][n_keys][n][2]: (qx qy qz qw), (tx ty tz theta); theta's sign
                              // bit: the next key lies on the other hemisphere
@@ -94,8 +108,9 @@ constexpr int kStatusTimeout = 4;
 
 constexpr uint32_t kJStart = 1u << 16;  // joint opens its segment
 constexpr uint32_t kJLink = 1u << 17;   // the joint's segment hangs from a parent joint
-// 16-bit joint info (shared memory): segment (14 bits) | start | link.
-constexpr uint16_t kJ16Seg = 0x3FFFu, kJ16Start = 0x4000u, kJ16Link = 0x8000u;
+// 16-bit joint info (shared memory): segment (13 bits) | the segment's prefix
+// ends in the odd buffer (pass2_qt) | start | link.
+constexpr uint16_t kJ16Seg = 0x1FFFu, kJ16Odd = 0x2000u, kJ16Start = 0x4000u, kJ16Link = 0x8000u;
 
 // One unit of work: `count` characters of one type.  For the frame the
 // characters share the key index k0 (so they read the same key records).

@@ -34,7 +34,45 @@ struct Segments {
   std::vector<int32_t> start, link;
   std::vector<uint16_t> seg_of;
   std::vector<uint32_t> jinfo;     // per joint: segment | kJStart | kJLink
+  // the prefix over the segment tree (TypeDev::hang, jump), and how many
+  // steps after the first each segment takes part in
+  std::vector<uint2> hang;
+  std::vector<uint32_t> jump;
+  std::vector<uint16_t> jump_n;
+  std::vector<int> steps;
 };
+
+// TypeDev::hang and jump of a segment decomposition.
+void build_jumps(Segments &S) {
+  std::vector<int> links(S.nseg, 0), up(S.nseg, -1), order;  // up: the segment the next link lies in
+  S.steps.assign(S.nseg, 0);
+  for (int g = 0; g < S.nseg; ++g) {
+    if (S.link[g] < 0) continue;
+    up[g] = S.seg_of[S.link[g]];
+    links[g] = links[up[g]] + 1;  // parents have smaller indices
+    while ((2 << S.steps[g]) < links[g]) ++S.steps[g];
+    order.push_back(g);
+  }
+  for (int g : order) {
+    const int second = S.link[up[g]];
+    S.hang.push_back(make_uint2((uint32_t)g | (uint32_t)S.link[g] << 16, second < 0 ? 0xFFFFFFFFu : (uint32_t)second));
+  }
+  std::vector<int> far(up);  // the segment 2^r links up
+  for (int r = 1;; ++r) {
+    std::vector<int> nxt(S.nseg, -1);
+    for (int g = 0; g < S.nseg; ++g) nxt[g] = far[g] < 0 ? -1 : far[far[g]];
+    far.swap(nxt);
+    int m = 0;
+    for (int g : order) {
+      if (S.steps[g] < r) continue;  // links <= 2^r
+      const uint32_t odd = (uint32_t)std::min(S.steps[far[g]], r - 1) & 1u;
+      S.jump.push_back((uint32_t)g | (uint32_t)far[g] << 12 | odd << 24);
+      ++m;
+    }
+    if (m == 0) break;
+    S.jump_n.push_back((uint16_t)m);
+  }
+}
 
 // Segments: maximal runs of consecutive joints where each joint's parent is
 // the previous joint (natural chains), each cut into ceil(m / seg_len)
@@ -78,6 +116,7 @@ Segments analyze_segments(const std::vector<int32_t> &par, int seg_len) {
     const int g = S.seg_of[j];
     S.jinfo[j] = (uint32_t)g | (j == S.start[g] ? kJStart : 0u) | (S.link[g] >= 0 ? kJLink : 0u);
   }
+  build_jumps(S);
   return S;
 }
 
@@ -475,7 +514,8 @@ struct TypeHost {
     std::vector<int16_t> s16(n), p16(n), g16(n);
     for (int j = 0; j < n; ++j) {
       const uint32_t i = seg.jinfo[j];
-      j16[j] = (uint16_t)((i & kJ16Seg) | ((i & kJStart) ? kJ16Start : 0u) | ((i & kJLink) ? kJ16Link : 0u));
+      j16[j] = (uint16_t)((i & kJ16Seg) | ((i & kJStart) ? kJ16Start : 0u) | ((i & kJLink) ? kJ16Link : 0u) |
+                          (seg.steps[seg.seg_of[j]] & 1 ? kJ16Odd : 0u));
       s16[j] = (int16_t)dfsord.sub_end[j];
       p16[j] = (int16_t)parent[j];
       g16[j] = (int16_t)(gather.empty() ? j : gather[j]);
@@ -484,6 +524,8 @@ struct TypeHost {
     const size_t o_s16 = B.add(s16.data(), s16.size() * 2);
     const size_t o_p16 = B.add(p16.data(), p16.size() * 2);
     const size_t o_g16 = B.add(g16.data(), g16.size() * 2);
+    const size_t o_hang = B.add(seg.hang.data(), seg.hang.size() * sizeof(uint2));
+    const size_t o_jump = B.add(seg.jump.data(), seg.jump.size() * 4);
     const size_t o_wt = B.add(ws.tab.data(), ws.tab.size() * 4);
     std::vector<int32_t> blk_out(n);
     for (int j = 0; j < n; ++j) {  // parent of the block-local root of j
@@ -514,6 +556,11 @@ struct TypeHost {
     dev.inv_gather = inv_gather.empty() ? nullptr : (const int32_t *)(base + o_ig);
     dev.jinfo = (const uint32_t *)(base + o_ji);
     dev.jinfo16 = (const uint16_t *)(base + o_j16);
+    dev.hang = (const uint2 *)(base + o_hang);
+    dev.jump = (const uint32_t *)(base + o_jump);
+    dev.n_hang = (int)seg.hang.size();
+    dev.n_jumps = (int)seg.jump_n.size();
+    std::copy(seg.jump_n.begin(), seg.jump_n.end(), dev.jump_n);
     dev.sub16 = (const int16_t *)(base + o_s16);
     dev.par16 = (const int16_t *)(base + o_p16);
     dev.gat16 = (const int16_t *)(base + o_g16);

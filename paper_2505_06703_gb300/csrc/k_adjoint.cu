@@ -198,9 +198,10 @@ __device__ __forceinline__ void adjoint_item(const AdjointArgs &a, const ItemBuf
   }
   cp_async_wait_all();  // this thread's table copies (adjoint_tables)
   pass_sync<NT>();
+  const Entry<uint2> first = pass2_first(b, tid);
   pass1b_qt<NT>(b, Lt, P, cs2, tid);
   pass_sync<NT>();
-  const float4 *Y = pass2_qt<NT>(b, Lt, P, cs2, tid);
+  pass2_qt<NT>(b, Lt, P, cs2, tid, first);
 
   // ---- model poses in place and the per-slot terms (g, p x g) in the same
   // pass; loss terms in F.w; slot n of each character is zero
@@ -210,7 +211,8 @@ __device__ __forceinline__ void adjoint_item(const AdjointArgs &a, const ItemBuf
     float4 *Pc = P + c * cs2;
     float3 p;
     if (info & kJ16Link) {
-      const QT m = qt_mul(lds_qt(Y, c * nseg + (int)(info & kJ16Seg), C * nseg), lds_qt(Pc, j, n));
+      const QT m = qt_mul(
+          lds_qt(info & kJ16Odd ? Lt.Y1 : Lt.Y0, c * nseg + (int)(info & kJ16Seg), C * nseg), lds_qt(Pc, j, n));
       sts_qt(Pc, j, n, m);
       p = make_float3(m.t.x, m.t.y, m.t.z);
     } else {

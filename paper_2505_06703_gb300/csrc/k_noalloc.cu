@@ -27,7 +27,7 @@ constexpr int kNoAllocSegLen = 16;
 
 // Scratch layout (byte offsets inside g_noalloc_scratch).
 constexpr size_t kOffType = 0;  // TypeDev
-constexpr size_t kOffQueue = 256;
+constexpr size_t kOffQueue = 448;
 constexpr size_t kOffParent = 512;
 constexpr size_t kOffSegStart = kOffParent + 4 * ANIM_MAX_JOINTS;
 constexpr size_t kOffSegLink = kOffSegStart + 4 * (ANIM_MAX_JOINTS + 64);

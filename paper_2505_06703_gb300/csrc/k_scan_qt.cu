@@ -203,28 +203,25 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
       const int W = n * b.cgroups, cpt = b.cpt;
       for (int idx = tid; idx < W; idx += kComputeThreads) {
         const int grp = (int)b.divN.div(idx), j = idx - grp * n;
-        const float4 qa0 = __ldg(KA0 + 2 * j), ta0 = __ldg(KA0 + 2 * j + 1);
-        const float4 qa1 = __ldg(KA1 + 2 * j), ta1 = __ldg(KA1 + 2 * j + 1);
-        float4 qb0 = qa0, tb0 = ta0, qb1 = qa1, tb1 = ta1;
+        const Key a0 = ldg_key(KA0 + 2 * j), a1 = ldg_key(KA1 + 2 * j);
+        Key b0 = a0, b1 = a1;
         if (two) {
-          qb0 = __ldg(KB0 + 2 * j);
-          tb0 = __ldg(KB0 + 2 * j + 1);
-          qb1 = __ldg(KB1 + 2 * j);
-          tb1 = __ldg(KB1 + 2 * j + 1);
+          b0 = ldg_key(KB0 + 2 * j);
+          b1 = ldg_key(KB1 + 2 * j);
         }
         const int c1 = min(C, (grp + 1) * cpt);
         for (int c = grp * cpt; c < c1; ++c) {
           const float al = b.alpha[c];
-          float4 q = slerp_pre(qa0, qa1, ta0.w, al);
-          float tx = fmaf(al, ta1.x - ta0.x, ta0.x), ty = fmaf(al, ta1.y - ta0.y, ta0.y),
-                tz = fmaf(al, ta1.z - ta0.z, ta0.z);
+          float4 q = slerp_pre(a0.q, a1.q, a0.t.w, al);
+          float tx = fmaf(al, a1.t.x - a0.t.x, a0.t.x), ty = fmaf(al, a1.t.y - a0.t.y, a0.t.y),
+                tz = fmaf(al, a1.t.z - a0.t.z, a0.t.z);
           if (two) {
-            const float4 qb = slerp_pre(qb0, qb1, tb0.w, al);
+            const float4 qb = slerp_pre(b0.q, b1.q, b0.t.w, al);
             const float w = b.blend[c];
             q = slerp_unit(q, qb, w);
-            tx = fmaf(w, fmaf(al, tb1.x - tb0.x, tb0.x) - tx, tx);
-            ty = fmaf(w, fmaf(al, tb1.y - tb0.y, tb0.y) - ty, ty);
-            tz = fmaf(w, fmaf(al, tb1.z - tb0.z, tb0.z) - tz, tz);
+            tx = fmaf(w, fmaf(al, b1.t.x - b0.t.x, b0.t.x) - tx, tx);
+            ty = fmaf(w, fmaf(al, b1.t.y - b0.t.y, b0.t.y) - ty, ty);
+            tz = fmaf(w, fmaf(al, b1.t.z - b0.t.z, b0.t.z) - tz, tz);
           }
           sts_qt(P + c * cs, j, n, QT{q, make_float4(tx, ty, tz, 0.f)});
         }
@@ -239,13 +236,13 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
     // chains 54.2 -> 43.8 us per frame; the forward on config 2, whose
     // 1,024-joint dragon it would also take, 50.6 -> 51.3 us)
     const bool chain = b.T.chain && C == 1 && n > 1024;
-    const float4 *Y = nullptr;
     if (chain) {
       chain_scan_qt(n, P, wtot, tid);
     } else {
+      const Entry<uint2> first = pass2_first(b, tid);
       pass1b_qt(b, Lt, P, cs, tid);
       compute_sync();
-      Y = pass2_qt(b, Lt, P, cs, tid);
+      pass2_qt(b, Lt, P, cs, tid, first);
     }
 
     // ---- pass 3: model pose, normalize, matrix, (bind,) store
@@ -263,7 +260,8 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
         const int c1 = min(C, (grp + 1) * cpt);
         for (int c = grp * cpt; c < c1; ++c) {
           QT m = lds_qt(P + c * cs, j, n);
-          if (!chain && (info & kJ16Link)) m = qt_mul(lds_qt(Y, c * nseg + g, C * nseg), m);
+          if (!chain && (info & kJ16Link))
+            m = qt_mul(lds_qt(info & kJ16Odd ? Lt.Y1 : Lt.Y0, c * nseg + g, C * nseg), m);
           const Aff M = aff_from_qt(normalize4(m.q), m.t.x, m.t.y, m.t.z);
           if (model) stg_aff(model4 + (b.off[c] + j) * 3, M);
           if (MODE == 3) {  // the joint's own slots: nobody else reads them in this pass
