@@ -836,7 +836,7 @@ struct anim_plan {
   std::vector<int> used;                      // type ids, most costly first
   std::vector<std::vector<int32_t>> by_type;  // characters of each used type (indexed like used)
   std::vector<int> C_skin, C_adj;             // per ctx type id
-  std::vector<int> C_frame;                   // plain frame: characters per (q, t) item
+  std::vector<int> C_fwd, C_frame, C_layers;  // (q, t) items: forward from local poses, plain frame, layers
   int64_t total = 0;
   int version = -1;  // schedule version the items were built for
   // device
@@ -855,7 +855,7 @@ struct anim_plan {
   int32_t *d_used = nullptr, *d_cap = nullptr;
   LaunchCfg cfg_scan{}, cfg_adj{};
   size_t smem_frame = 0;     // plain frame, (q, t) items
-  size_t smem_skin = 0;      // frame with skinning
+  size_t smem_skin = 0, smem_layers = 0;  // frames with skinning, with layered blending
   int adj_unfit = -1;
   // frame: item slots [0, n_slots_walk) belong to the chain-walk kernel
   // (queue counters d_queue[0..1]), the rest to the segmented CTA kernel
@@ -1013,12 +1013,15 @@ size_t adj_budget(const anim_ctx *ctx) {
   return ctx->smem_per_sm / (size_t)ctx->adj_ctas - 1024 - kAdjSmallStatic;
 }
 
-// Characters per work item: kind 0 the matrix scan, 1 the adjoint, 2 the
-// plain frame's (q, t) items, 3 the frame with skinning's.
-int choose_C(const anim_ctx *ctx, const TypeHost &T, int kind) {
+// Resident CTAs the adjoint's items are taken by.
+int adj_slots(const anim_ctx *ctx) { return ctx->sm_count * (ctx->adj_ctas > 0 ? ctx->adj_ctas : ctx->ctas_per_sm); }
+
+// Characters per work item of `target` joints: kind 0 the matrix scan, 1 the
+// adjoint, 2 the plain frame's (q, t) items, 3 the frame with skinning's.
+int choose_C(const anim_ctx *ctx, const TypeHost &T, int kind, int target) {
   const bool adjoint = kind == 1;
   const size_t budget = adjoint ? adj_budget(ctx) : smem_budget(ctx);
-  int C = std::max(1, std::min(kCMax, ctx->joints_per_item / std::max(1, T.n)));
+  int C = std::max(1, std::min(kCMax, target / std::max(1, T.n)));
   auto bytes = [&](int c) {
     return kind == 1   ? adjoint_smem_bytes(T.n, T.seg.nseg, c)
            : kind == 2 ? scan_qt_smem_bytes(T.n, T.seg.nseg, c)
@@ -1028,6 +1031,48 @@ int choose_C(const anim_ctx *ctx, const TypeHost &T, int kind) {
   while (C > 1 && bytes(C) > budget) --C;
   if (bytes(C) > ctx->smem_optin - kStaticSmemAllowance) return 0;
   return C;
+}
+
+// Item size in joints for a batch: the schedule's or, where that fills the
+// resident CTAs (`slots`) less than kBalanceWaves times over, the smallest
+// whose items still go round in as many waves.  A CTA takes its items'
+// passes one after the other, so a small batch in few large items leaves the
+// chip idle, and a second wave of a few large items takes as long as the
+// first: the forward of 64 characters of 64 joints as two items of 32 took
+// 10.9 us, as 64 items 6.2; 1,000 of them 11.3 and 7.8; the skinned frame of
+// 304 22.1 and 12.5.  From a few waves on the sizes meet (3,000 of 300
+// joints, 9 waves: 34.7 both ways).  `binned`: work items that the frame's
+// queue forms per key index; each non-empty bin of a range then ends with a
+// part-filled item, (C - 1) / 2C of one on average.
+constexpr int kBalanceWaves = 3;
+struct BatchType {
+  const TypeHost *T;
+  int64_t chars;
+};
+int item_target(const anim_ctx *ctx, const std::vector<BatchType> &batch, int slots, int kind, bool binned) {
+  auto items = [&](int target) {
+    double n = 0.0;
+    for (const BatchType &t : batch) {
+      const int C = std::max(1, choose_C(ctx, *t.T, kind, target));
+      if (binned) {
+        const double bins = (double)std::min<int64_t>(
+            t.chars, (t.chars + kRangeChars - 1) / kRangeChars * std::max(1, std::min(t.T->n_keys, kRangeChars)));
+        n += (double)t.chars / C + bins * (C - 1) / (2.0 * C);
+      } else {
+        n += (double)((t.chars + C - 1) / C);
+      }
+    }
+    return n;
+  };
+  int lo = 1, hi = ctx->joints_per_item;
+  const double waves = std::ceil(items(hi) / slots);
+  if (waves > kBalanceWaves) return hi;
+  while (lo < hi) {  // items() falls as the target grows
+    const int mid = (lo + hi) / 2;
+    if (items(mid) <= waves * slots) hi = mid;
+    else lo = mid + 1;
+  }
+  return hi;
 }
 
 template <class T>
@@ -1065,20 +1110,35 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   const int nt = (int)ctx->types.size();
   P->C_skin.assign(nt, 1);
   P->C_adj.assign(nt, 1);
-  P->C_frame.assign(nt, 1);
+  for (auto *v : {&P->C_fwd, &P->C_frame, &P->C_layers}) v->assign(nt, 1);
   P->adj_unfit = -1;
-  size_t smem_s = 0, smem_a = 0, smem_q = 0;
+  size_t smem_s = 0, smem_a = 0, smem_q = 0, smem_l = 0;
+  std::vector<BatchType> all, adj, seg;  // every type, its adjoint view, the types off the walk kernel
+  for (size_t u = 0; u < P->used.size(); ++u) {
+    const TypeHost &T = *ctx->types[P->used[u]];
+    const int64_t cnt = (int64_t)P->by_type[u].size();
+    all.push_back({&T, cnt});
+    adj.push_back({T.adj.get(), cnt});
+    if (!ctx->use_walk || !T.walk_ready()) seg.push_back({&T, cnt});
+  }
+  const int ctas = ctx->sm_count * ctx->ctas_per_sm;
+  const int t_fwd = item_target(ctx, all, ctas, 2, false), t_frame = item_target(ctx, seg, ctas, 2, true),
+            t_layers = item_target(ctx, all, ctas, 2, true), t_skin = item_target(ctx, all, ctas, 3, true),
+            t_adj = item_target(ctx, adj, adj_slots(ctx), 1, false);
   for (int t : P->used) {
     const TypeHost &T = *ctx->types[t];
-    const int cs = choose_C(ctx, T, 0), ca = choose_C(ctx, *T.adj, 1);
+    const int cs = choose_C(ctx, T, 0, 1), ca = choose_C(ctx, *T.adj, 1, t_adj);
     if (cs == 0)
       return fail(ctx, ANIM_EUNSUPPORTED,
                   "type %d (%d joints, %d segments) does not fit in shared memory with one character", t, T.n,
                   T.seg.nseg);
-    P->C_frame[t] = std::max(cs, choose_C(ctx, T, 2));  // (q, t) items are smaller
-    P->C_skin[t] = std::max(cs, choose_C(ctx, T, 3));
+    P->C_fwd[t] = choose_C(ctx, T, 2, t_fwd);
+    P->C_frame[t] = choose_C(ctx, T, 2, t_frame);
+    P->C_layers[t] = choose_C(ctx, T, 2, t_layers);
+    P->C_skin[t] = choose_C(ctx, T, 3, t_skin);
     smem_s = std::max(smem_s, scan_skin_smem_bytes(T.n, T.seg.nseg, P->C_skin[t]));
-    smem_q = std::max(smem_q, scan_qt_smem_bytes(T.n, T.seg.nseg, P->C_frame[t]));
+    smem_q = std::max(smem_q, scan_qt_smem_bytes(T.n, T.seg.nseg, P->C_fwd[t]));
+    smem_l = std::max(smem_l, scan_qt_smem_bytes(T.n, T.seg.nseg, P->C_layers[t]));
     // the adjoint keeps two more vectors per joint: a schedule may fit the
     // forward kernels and not the adjoint, which then refuses to run
     if (ca == 0) {
@@ -1089,7 +1149,7 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
     smem_a = std::max(smem_a, adjoint_smem_bytes(T.adj->n, T.adj->seg.nseg, ca));
   }
   // static items: (q, t) items for the forward from local poses, adjoint items
-  auto is = make_items(P, P->C_frame), ia = make_items(P, P->C_adj);
+  auto is = make_items(P, P->C_fwd), ia = make_items(P, P->C_adj);
   P->n_items_scan = (int)is.size();
   P->n_items_adj = (int)ia.size();
   CK(upload_vec(&P->d_items_scan, is));
@@ -1167,7 +1227,7 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
     return sl;
   };
   std::vector<RangeDev> ranges_cta, ranges_qa;
-  const int slots_cta = all_types(P->C_skin, ranges_cta), slots_qa = all_types(P->C_frame, ranges_qa);
+  const int slots_cta = all_types(P->C_skin, ranges_cta), slots_qa = all_types(P->C_layers, ranges_qa);
   P->n_ranges_cta = (int)ranges_cta.size();
   P->n_slots_cta = slots_cta;
   CK(upload_vec(&P->d_ranges_cta, ranges_cta));
@@ -1175,7 +1235,7 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   P->n_ranges_qa = (int)ranges_qa.size();
   P->n_slots_qa = slots_qa;
   CK(upload_vec(&P->d_ranges_qa, ranges_qa));
-  CK(upload_vec(&P->d_cap_qa, P->C_frame));
+  CK(upload_vec(&P->d_cap_qa, P->C_layers));
   P->vert_off.assign(P->n_chars + 1, 0);
   for (int64_t c = 0; c < P->n_chars; ++c)
     P->vert_off[c + 1] = P->vert_off[c] + ctx->types[P->char_type[c]]->n_verts;
@@ -1193,6 +1253,7 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
                   ctx->ctas_per_sm >= 3 ? 3 : 2};
   P->smem_frame = std::max<size_t>(smem_f, 16);
   P->smem_skin = std::max<size_t>(smem_s, 16);
+  P->smem_layers = std::max<size_t>(smem_l, 16);
   P->version = ctx->version;
   return ANIM_OK;
 }
@@ -1846,8 +1907,9 @@ int anim_evaluate_frame_layers(anim_ctx *ctx, const anim_plan *plan, const float
   a.skin = d_skin;
   a.layer_w = d_weights;
   a.add_w = d_add_w;
-  LaunchCfg cfg = plan->cfg_scan;  // its shared memory covers every type's (q, t) item
-  cfg.ctas = ctx->sm_count * ctx->ctas_per_sm;
+  LaunchCfg cfg = plan->cfg_scan;
+  cfg.ctas = std::max(1, std::min(ctx->sm_count * ctx->ctas_per_sm, a.n_items));
+  cfg.smem = plan->smem_layers;
   CK(launch_scan_qt(2, a, cfg, (cudaStream_t)stream));
   return ANIM_OK;
 }
@@ -2029,11 +2091,18 @@ int anim_ik_create(anim_ctx *ctx, const anim_plan *plan, int n_eff, const int32_
     CK(ev);
     for (int e = 0; e < n_eff; ++e) eff_slot[(size_t)t * n_eff + e] = vid[effectors[(size_t)t * n_eff + e]];
     vdev[t] = V->dev;
-    const int C = choose_C(ctx, *V, 1);
+    K->views[t] = std::move(V);
+  }
+  std::vector<BatchType> batch;
+  for (size_t u = 0; u < plan->used.size(); ++u)
+    batch.push_back({K->views[plan->used[u]].get(), (int64_t)plan->by_type[u].size()});
+  const int target = item_target(ctx, batch, adj_slots(ctx), 1, false);
+  for (int t : plan->used) {
+    const TypeHost &V = *K->views[t];
+    const int C = choose_C(ctx, V, 1, target);
     if (C == 0) return fail(ctx, ANIM_EUNSUPPORTED, "IK view of type %d does not fit in shared memory", t);
     Cv[t] = C;
-    smem = std::max(smem, adjoint_smem_bytes(V->n, V->seg.nseg, C));
-    K->views[t] = std::move(V);
+    smem = std::max(smem, adjoint_smem_bytes(V.n, V.seg.nseg, C));
   }
   CK(upload_vec(&K->d_views, vdev));
   CK(upload_vec(&K->d_eff, eff_slot));
