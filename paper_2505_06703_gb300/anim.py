@@ -62,6 +62,7 @@ SIGNATURES = {
 }
 
 _lib = None
+_torch_c = None  # torch's C module, set by the first Context
 
 
 def lib_path() -> str:
@@ -95,20 +96,23 @@ def _np_ptr(a):
 
 
 def _dptr(t):
-    """Device pointer of a CUDA tensor (or None)."""
+    """Device pointer of a CUDA tensor (or None), as the integer ctypes takes for a void *."""
     if t is None:
         return None
     if not t.is_cuda:
         raise ValueError("expected a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError("expected a contiguous tensor")
-    return c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream=None):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return c_void_p(s.cuda_stream)
+    """Handle of the given stream, or of the current device's current stream
+    (read without building a torch.cuda.Stream, which takes 3 us of a call
+    that issues in 10)."""
+    if stream is not None:
+        return stream.cuda_stream
+    return _torch_c._cuda_getCurrentRawStream(_torch_c._cuda_getDevice())
 
 
 def analyze_skeleton(parents, seg_len: int = 8):
@@ -129,9 +133,12 @@ class Context:
 
     def __init__(self, device: int = 0):
         import torch
+        global _torch_c
         self.lib = load()
         self.device = device
         torch.cuda.init()
+        _torch_c = torch._C
+        self._empty, self._f32, self._dev = torch.empty, torch.float32, torch.device("cuda", int(device))
         h = c_void_p()
         rc = self.lib.anim_create(ctypes.byref(h), int(device))
         if rc != ANIM_OK:
@@ -242,10 +249,7 @@ class Context:
 
     # ---------------------------------------------------------- evaluation
     def _out(self, plan, cols, out):
-        import torch
-        if out is None:
-            out = torch.empty((plan.total, cols), dtype=torch.float32, device=f"cuda:{self.device}")
-        return out
+        return self._empty((plan.total, cols), dtype=self._f32, device=self._dev) if out is None else out
 
     def evaluate_frame(self, plan, time, blend_w, out=None, stream=None, levelsync=False):
         """Fused frame: skin matrices [total, 12] from per-character time and blend weight."""
@@ -309,11 +313,10 @@ class Context:
         return grad_q, grad_t
 
     def loss_backward(self, plan, q, t, target, grad_q=None, grad_t=None, loss=None, stream=None):
-        import torch
         grad_q = self._out(plan, 4, grad_q)
         grad_t = self._out(plan, 3, grad_t)
         if loss is None:
-            loss = torch.empty(plan.n_chars, dtype=torch.float32, device=f"cuda:{self.device}")
+            loss = self._empty(plan.n_chars, dtype=self._f32, device=self._dev)
         self._ck(self.lib.anim_loss_backward(self.h, plan.h, _dptr(q), _dptr(t), _dptr(target), _dptr(grad_q),
                                              _dptr(grad_t), _dptr(loss), _stream(stream)))
         return grad_q, grad_t, loss
@@ -404,7 +407,7 @@ def hierarchy_fn():
             _, model = actx.forward_local(plan, q, t, skin=False, model=True)
             fctx.save_for_backward(q, t)
             fctx.actx, fctx.plan = actx, plan
-            return model.view(-1, 3, 4)[:, :, 3]
+            return model[:, 3::4]  # the translation column of each 3x4 matrix
 
         @staticmethod
         def backward(fctx, grad_pos):
