@@ -61,7 +61,7 @@ NCU_TRAFFIC = {"9d28c9fadbd4aae7": 2654464 + 42383616}
 
 # ------------------------------------------------------------------ helpers
 # The sources the persistent frame kernel is compiled and launched from.
-FRAME_KERNEL_SOURCES = ("anim_internal.h", "dev_math.cuh", "scan_core.cuh", "k_scan_qt.cu", "k_walk.cu", "k_walk2.cu",
+FRAME_KERNEL_SOURCES = ("anim_internal.h", "dev_math.cuh", "scan_core.cuh", "k_scan_qt.cu", "k_walk2.cu",
                         "smem_limit.h", "host.cu")
 
 
@@ -375,8 +375,7 @@ def run_ours(args) -> dict:
     tr = NCU_TRAFFIC.get(kernel_source_hash())
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": tr,
-                "kernel": {0: "k_scan_qt<0> (persistent frame)", 1: "k_walk (chain walk in skin space)",
-                           2: "k_walk2 (warp-specialized chain walk in skin space)"}[schedule[3]],
+                "kernel": "k_walk2 (chain walk in skin space)" if schedule[3] else "k_scan_qt<0> (persistent frame)",
                 "kernel_ms": round(k_ms, 5), "algorithmic_bytes": alg, "peak_source": peak_src,
                 "nominal_peak": NOMINAL_HBM_GBS, "frac_of_nominal": round(achieved / NOMINAL_HBM_GBS, 4),
                 "touched_bytes": frame_touched_bytes(w)}

@@ -69,7 +69,7 @@ struct TypeDev {
   int n_faces;
   const float4 *mesh;
   const int32_t *faces;      // [n_faces][3] vertex indices (raster)
-  // Chain-walk frame kernel (k_walk): a static lane schedule of wk_S steps
+  // Chain-walk frame kernel (k_walk2): a static lane schedule of wk_S steps
   // for wk_P lanes per character, staged in chunks of wk_K steps (the table
   // is padded with idle entries to whole chunks); entry [s][slot] names the
   // joint lane `slot` composes at step s (kWInvalid: idle).  wk_mode 1:
@@ -96,7 +96,7 @@ constexpr int kWLoadShift = 15;             // bits 15-22
 constexpr int kWStoreShift = 23;            // bits 23-30
 constexpr uint32_t kWRootSlot = 255;        // load slot of a chain that starts at a root
 constexpr int kWalkMaxSteps = 160;          // longest schedule the walk kernel takes (latency bound)
-constexpr int kWalkMaxSmem = 32 * 1024;     // shared memory of one walk CTA (staging + branch slots)
+constexpr int kWalkMaxBranch = 18560;       // bytes of branch-point slots of a walk item
 // Static shared memory the persistent kernels may use besides the dynamic
 // item buffers (two staged work items, scan scratch); the host subtracts it
 // from the per-CTA budget.
@@ -242,7 +242,8 @@ struct AdjointArgs {
 };
 cudaError_t launch_adjoint(int mode, const AdjointArgs &a, const LaunchCfg &cfg, cudaStream_t s);
 
-// Chain-walk frame kernel: one-warp CTAs, CTA i running work-queue slot i
+// Chain-walk frame kernel (three warps per item: two sample and write out,
+// one walks), CTA i running work-queue slot i
 // (at most 32 / wk_P characters of one walk type sharing the key index k0;
 // empty slots exit), composing them lane-parallel along the type's schedule.
 struct WalkArgs {
@@ -256,16 +257,13 @@ struct WalkArgs {
   const float *time, *blend_w;
   float *skin;
   // 0: wait for the preceding grid (the work-queue kernel) before reading
-  // the item.  1 (k_walk2 only): the preceding grid is the segmented frame
+  // the item.  1: the preceding grid is the segmented frame
   // kernel, which lets this launch start only after its own wait for the
   // work queue; the item and the inputs are read from L2 at once, and each
   // CTA waits for that grid at its end, so that the next launch in the
   // stream (the next frame's work queue) still follows both.
   int pred_waited;
 };
-size_t walk_smem_bytes(int chars_per_item, int nbs);
-// The warp-specialized variant (three warps per item: two sample and write
-// out, one walks), same arguments and tables.
 size_t walk2_smem_bytes(int chars_per_item, int nbs);
 cudaError_t launch_walk2(const WalkArgs &a, size_t smem, cudaStream_t s);
 int walk2_blocks_per_sm(size_t smem);
@@ -274,8 +272,6 @@ int walk2_blocks_per_sm(size_t smem);
 // block scheduler then spreads the items evenly instead of stacking one
 // more on some SMs (the frame ends with its most loaded SM).
 size_t walk2_spread_smem(size_t smem, int n_items, int sm_count);
-cudaError_t launch_walk(const WalkArgs &a, size_t smem, cudaStream_t s);
-int walk_blocks_per_sm(size_t smem);  // resident one-warp CTAs per SM at this shared-memory size
 
 // The paper's Algorithms 1-4 (comparators): one CTA per character.
 constexpr int kPaperMaxJoints = 1024;

@@ -340,7 +340,7 @@ WalkSched choose_walk(const std::vector<int32_t> &par) {
   for (int P = 1; P <= 32; P *= 2) {
     WalkSched W = walk_tree(par, P);
     if (W.mode == 0 || W.S > kWalkMaxSteps) continue;
-    if (walk_smem_bytes(32 / P, W.nbs) > kWalkMaxSmem) continue;
+    if (48 * (32 / P) * W.nbs > kWalkMaxBranch) continue;
     if (!walk_check(W, par)) continue;
     best = std::max(best, (double)n / ((double)W.S * P));
     cand.push_back(std::move(W));
@@ -931,8 +931,8 @@ struct anim_ctx {
   int *d_status = nullptr;
   int version = 0;  // bumps when types/schedules change
   int ctas_per_sm = 2;            // resident persistent CTAs per SM the schedule is sized for
-  int use_walk = 1;               // frame: walkable types run on the chain-walk kernel (2: its
-                                  // warp-specialized variant)
+  int use_walk = 1;               // frame: walkable types run on the chain-walk kernel (nonzero;
+                                  // two values from when it had two variants)
   int adj_ctas = 0;               // adjoint: 0 = persistent kernel, k = one-item kernel sized for k CTAs per SM
   cudaStream_t side = nullptr;    // frame: the CTA kernel's stream when both kernels have work
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -1103,6 +1103,34 @@ std::vector<WorkItem> make_items(const anim_plan *P, const std::vector<int> &Cv)
   return items;
 }
 
+// Whether the plan's walkable types run on the chain-walk kernel under a
+// schedule that allows it.  The walk's time is its longest schedule's, S
+// steps whatever the batch, until its warps fill the chip; the segmented
+// kernel's is a short item's, then grows with the joints, and a joint costs
+// it more.  So the walk needs a batch, the larger the longer the schedule.
+// Measured, us on the segmented kernel / the walk:
+//   67 joints, S about 16: 41 thousand joints 10.7/10.8, 67 thousand
+//     11.6/11.5, 134 thousand 14.4/12.5;
+//   ragged 200, 126, 53 joints, S about 40: 126 thousand 14.0/20.9, 250
+//     thousand 20.0/22.5, 500 thousand 30.4/27.9;
+//   300 joints, S about 64: 12 thousand 11.5/23.6, 300 thousand 20.4/28.0,
+//     600 thousand 33.0/32.7, 1.2 million 56.9/42.2;
+//   512-joint bipeds, S about 70: 0.5 million 20.8/27.6, 1.0 million
+//     33.7/32.7, 2.1 million 57.6/47.7.
+// 165 S^2 joints lie on or a little below where each pair meets.
+constexpr int64_t kWalkJointsPerStep2 = 165;
+bool walk_pays(const anim_ctx *ctx, const anim_plan *P) {
+  if (!ctx->use_walk) return false;
+  int64_t joints = 0, S = 0;
+  for (size_t u = 0; u < P->used.size(); ++u) {
+    const TypeHost &T = *ctx->types[P->used[u]];
+    if (!T.walk_ready()) continue;
+    joints += (int64_t)T.n * (int64_t)P->by_type[u].size();
+    S = std::max<int64_t>(S, T.ws.S);
+  }
+  return joints >= kWalkJointsPerStep2 * S * S;
+}
+
 // (Re)build the schedule-dependent parts of a plan: characters per item,
 // static items, launch configurations.
 int plan_schedule(anim_ctx *ctx, anim_plan *P) {
@@ -1113,13 +1141,15 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   for (auto *v : {&P->C_fwd, &P->C_frame, &P->C_layers}) v->assign(nt, 1);
   P->adj_unfit = -1;
   size_t smem_s = 0, smem_a = 0, smem_q = 0, smem_l = 0;
+  const bool walks = walk_pays(ctx, P);
+  auto on_walk = [&](const TypeHost &T) { return walks && T.walk_ready(); };
   std::vector<BatchType> all, adj, seg;  // every type, its adjoint view, the types off the walk kernel
   for (size_t u = 0; u < P->used.size(); ++u) {
     const TypeHost &T = *ctx->types[P->used[u]];
     const int64_t cnt = (int64_t)P->by_type[u].size();
     all.push_back({&T, cnt});
     adj.push_back({T.adj.get(), cnt});
-    if (!ctx->use_walk || !T.walk_ready()) seg.push_back({&T, cnt});
+    if (!on_walk(T)) seg.push_back({&T, cnt});
   }
   const int ctas = ctx->sm_count * ctx->ctas_per_sm;
   const int t_fwd = item_target(ctx, all, ctas, 2, false), t_frame = item_target(ctx, seg, ctas, 2, true),
@@ -1163,7 +1193,7 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   P->walk_nbs = 0;
   for (int t : P->used) {
     const TypeHost &T = *ctx->types[t];
-    if (!ctx->use_walk || !T.walk_ready()) {
+    if (!on_walk(T)) {
       smem_f = std::max(smem_f, scan_qt_smem_bytes(T.n, T.seg.nseg, P->C_frame[t]));
       continue;
     }
@@ -1196,12 +1226,10 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
     }
     if (pass == 0) P->n_slots_walk = slots;
   }
-  const bool walk2 = ctx->use_walk == 2;
-  P->walk_smem = P->n_slots_walk == 0 ? 0 : walk2 ? walk2_smem_bytes(wcmax, P->walk_nbs)
-                                                   : walk_smem_bytes(wcmax, P->walk_nbs);
-  if (walk2 && P->n_slots_walk > 0) P->walk_smem = walk2_spread_smem(P->walk_smem, P->n_slots_walk, ctx->sm_count);
-  if (P->n_slots_walk > 0 &&
-      (walk2 ? walk2_blocks_per_sm(P->walk_smem) : walk_blocks_per_sm(P->walk_smem)) < 1)
+  P->walk_smem = 0;
+  if (P->n_slots_walk > 0)
+    P->walk_smem = walk2_spread_smem(walk2_smem_bytes(wcmax, P->walk_nbs), P->n_slots_walk, ctx->sm_count);
+  if (P->n_slots_walk > 0 && walk2_blocks_per_sm(P->walk_smem) < 1)
     return fail(ctx, ANIM_EUNSUPPORTED, "chain-walk kernel: no resident CTA at %zu bytes of shared memory",
                 P->walk_smem);
   P->n_ranges = (int)ranges.size();
@@ -1678,7 +1706,7 @@ int anim_frame_run_queue(anim_ctx *ctx, const anim_plan *plan, const float *d_ti
   // after it), and the next launch in the stream keeps a single kernel
   // predecessor -- a fork onto the side stream and back ends that chain and
   // costs the next frame its early start.
-  const bool chain = has_walk && has_cta && ctx->use_walk == 2 && plan->n_slots - plan->n_slots_walk <= kChainSlots;
+  const bool chain = has_walk && has_cta && plan->n_slots - plan->n_slots_walk <= kChainSlots;
   if (has_walk && has_cta && !chain) {
     // the two kernels run side by side: fork onto the context's side stream
     if (!ctx->side) {
@@ -1725,10 +1753,7 @@ int anim_frame_run_queue(anim_ctx *ctx, const anim_plan *plan, const float *d_ti
     w.blend_w = d_blend_w;
     w.skin = d_skin;
     w.pred_waited = chain ? 1 : 0;
-    if (ctx->use_walk == 2)
-      CK(launch_walk2(w, plan->walk_smem, st));
-    else
-      CK(launch_walk(w, plan->walk_smem, st));
+    CK(launch_walk2(w, plan->walk_smem, st));
   }
   if (has_walk && has_cta && !chain) {
     CK(cudaEventRecord(ctx->ev_join, ctx->side));
@@ -2251,7 +2276,7 @@ static void for_each_candidate(const anim_ctx *ctx, int which, F &&f) {
   const int adjs[] = {0, 4, 6, 7, 8};
   const int walk_lo = which == 0 ? 0 : ctx->use_walk, walk_hi = which == 0 ? 2 : ctx->use_walk;
   const int adj_keep = ctx->adj_ctas;
-  for (int walk = walk_lo; walk <= walk_hi; ++walk)
+  for (int walk = walk_lo; walk <= walk_hi; walk += 2)  // 1 and 2 run the same kernel
     for (int adj : adjs)
       for (int seg : segs)
         for (int cps : cpss)

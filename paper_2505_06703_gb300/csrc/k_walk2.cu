@@ -1,8 +1,29 @@
-// Warp-specialized chain walk (the frame, Sec. 1 steps 1-3, Eq. 1, in skin
-// space as in k_walk.cu): the same static lane schedule and bind-folded key
-// records, with the work of one item split over three warps so that the
-// sampling runs on more warps per SM than the walk's lanes alone provide and
-// the skin matrices leave as lane-contiguous stores:
+// Chain-walk frame kernel: Simulation -> Hierarchy-Scan -> Bind MeshPose
+// (Sec. 1 steps 1-3, Eq. 1) walked directly in skin space, for skeleton
+// types whose natural chains can be list-scheduled on a few lanes with few
+// idle steps (long pure chains stay on the segmented kernel).
+//
+// Skin-space walk.  With rigid inverse binds B, the skin matrix of joint j
+// satisfies S_j = M_j B_j = S_p (B_p^-1 L_j B_j) = S_p L'_j (p the parent; a
+// root has B_p = I).  Because slerp commutes with multiplying both of its
+// ends by unit quaternions on the left and on the right, and lerp with any
+// affine map, L'_j is sampled exactly like L_j from key records whose
+// rotations are q' = conj(q_Bp) q q_Bj and whose translations are
+// R_Bp^T (t - t_Bp); its translation then needs R' u_j with u_j = R_Bj^T t_Bj
+// (minus the joint's rest position).  The host builds these records once per
+// clip upload, so per joint and character the kernel samples two key pairs,
+// blends them, forms L' = [R(q') | t' + R(q') u] and makes ONE 3x4 product,
+// which is the skin matrix it stores -- no separate bind product, no second
+// pass over the joints, no block barrier.
+//
+// A work item is C = 32 / P characters of one type that share the key index
+// k0; lane = (character, schedule slot).  The type's static schedule (host-
+// built) names the joint each slot composes at each step.  A lane keeps S in
+// registers along its natural chain; branch points leave S in a shared-memory
+// slot for the lane that starts a child chain at a later step.  The work of
+// one item is split over three warps, so that the sampling runs on more warps
+// per SM than the walk's lanes alone provide and the skin matrices leave as
+// lane-contiguous stores:
 //   warps 1 and 2 (samplers)  wait for a chunk of key records staged by
 //       cp.async.bulk, sample the local rotation q' and translation t' of
 //       half of its steps each into the chunk's row buffer, and write the
@@ -83,9 +104,8 @@ __device__ __forceinline__ void rec_sample_w2(const float4 *r, int P, float al, 
   rec_eval(r[0], r[P], r[2 * P], r[3 * P], al, q, t);
 }
 // Shared memory of one CTA (dynamic, 128-byte aligned parts):
-//   rec[2]   staged key records, u and schedule entries of a chunk, the
-//            layout of k_walk's chunk buffer (clip 0 records [K][4][P],
-//            clip 1 records, u [K][P], entries [K][P])
+//   rec[2]   staged key records, u and schedule entries of a chunk (clip 0
+//            records [K][4][P], clip 1 records, u [K][P], entries [K][P])
 //   x[2]     the chunk's row buffer, kXStride(K) float4 per lane (an odd
 //            stride: lane-indexed accesses are free of bank conflicts): at
 //            3k, 3k+1 the samplers' transform of step k (q', then t' with
