@@ -181,7 +181,7 @@ ANIM_API int anim_evaluate_frame(anim_ctx *ctx, const anim_plan *plan, const flo
  * Page-locked buffers (cudaMallocHost, cudaHostRegister) make the copies
  * asynchronous; pageable ones work through the driver's staging.  A plan of
  * at least 1,024 characters is evaluated in up to 4 contiguous ranges of
- * nearly equal joint counts, each range's skin matrices copied back on a
+ * growing joint counts, each range's skin matrices copied back on a
  * second stream of the plan while the next range's frame runs (the call's
  * `stream` waits for those copies, so the rule above holds).  The device
  * staging buffers (n_chars x 8 B + total x 48 B), the ranges' own plans, the
