@@ -75,6 +75,11 @@ __device__ __forceinline__ Key ldg_key(const float4 *p) {
   return k;
 }
 
+// a + f (b - a) of the first three components.
+__device__ __forceinline__ float4 lerp_t(const float4 a, const float4 b, const float f) {
+  return make_float4(fmaf(f, b.x - a.x, a.x), fmaf(f, b.y - a.y, a.y), fmaf(f, b.z - a.z, a.z), 0.f);
+}
+
 // Weighted sum w0*a + w1*b followed by normalization.
 __device__ __forceinline__ float4 combine_norm(const float4 a, const float4 b, const float w0, const float w1) {
   float4 r;

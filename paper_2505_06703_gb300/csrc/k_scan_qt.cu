@@ -6,7 +6,7 @@
 //   MODE 1  the forward from given local poses q [total][4] (normalized
 //           here), t [total][3], skin and / or model matrices out;
 //   MODE 2  the frame with layered blending (up to 4 clips by per-character
-//           weights and an additive layer, sample_layers_at);
+//           weights and an additive layer, sample_layers);
 //   MODE 3  the plain frame followed by linear blend skinning: the bind pass
 //           leaves the skin matrices' rows in shared memory (a third plane
 //           beside q and t) for the skinning pass, and writes them to global
@@ -185,11 +185,10 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
         sts_qt(P + c * cs, j, n, QT{q, make_float4(__ldg(tp), __ldg(tp + 1), __ldg(tp + 2), 0.f)});
       }
     } else if (MODE == 2) {
-      // character-minor: the lanes of one joint share its key records
-      const int CN = C * n;
-      for (int idx = tid; idx < CN; idx += kComputeThreads) {
-        const int j = (int)b.divC.div(idx), c = idx - j * C;
-        sts_qt(P + c * cs, j, n, sample_layers_at(b, j, c));
+      const int W = n * b.cgroups, cpt = b.cpt;
+      for (int idx = tid; idx < W; idx += kComputeThreads) {
+        const int grp = (int)b.divN.div(idx), j = idx - grp * n;
+        sample_layers(b, j, grp * cpt, min(C, (grp + 1) * cpt), P, cs);
       }
     } else {
       const int nk = b.T.n_keys, k0 = b.k0, k1 = (k0 + 1 == nk) ? 0 : k0 + 1;
