@@ -185,7 +185,7 @@ __device__ __forceinline__ void w2_write_out(const float4 *xb, const uint32_t (&
     if (d == kNoPart) continue;
     const int src = d & 31, r = (d >> 5) & 15, k = (d >> 9) & 3;
     const uint32_t j = xj[(src * X + 3 * K) * 4 + k];
-    if (j != kWInvalid) outs[src >> logP][3 * j + (r - 3 * k)] = xb[src * X + r];
+    if (j != kWInvalid) __stcs(outs[src >> logP] + 3 * j + (r - 3 * k), xb[src * X + r]);  // as stg_aff
   }
 }
 
