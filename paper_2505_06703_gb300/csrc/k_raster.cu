@@ -195,7 +195,8 @@ __device__ __forceinline__ void test_pixel(const RasterArgs &a, const WarpTris &
 // the image, all three launches): 422 us with a triangle per lane in 64-bit
 // arithmetic from global vertices, 226 with staged vertices and 32-bit
 // edges, 176 with a row per lane, 112 as it is (83.8 M warp instructions at
-// 75 % issue; the vertices' 147 MB take 22 us).  A 5-CTA build spills: 116.
+// 75 % issue; the vertices' 147 MB take 22 us).  A 5-CTA build spills: 116;
+// three CTAs per SM: 122.
 __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_tris(const __grid_constant__ RasterArgs a) {
   extern __shared__ int2 sxy[];
   __shared__ WarpTris tris[kRasterThreads / 32];
