@@ -354,8 +354,9 @@ ANIM_API int anim_tune_ik(anim_ctx *ctx, anim_plan *plan, int n_eff, const int32
 /* The schedule the autotuner picked, as 5 integers: segment length, resident
  * CTAs per SM, work-item size in joints (an upper bound: a batch that does
  * not fill the chip at that size takes smaller items), chain-walk kernel for
- * the frame (0: none, 1 or 2: for walkable types in batches large enough that
- * it is the faster kernel), adjoint kernel (0: persistent, k = 1..8: one work item per CTA,
+ * the frame (0: never, 1: for every walkable type, 2, the default: for
+ * walkable types in batches large enough that it is the faster kernel;
+ * anim_plan_walk tells), adjoint kernel (0: persistent, k = 1..8: one work item per CTA,
  * items sized so k CTAs share an SM) -- read with anim_get_schedule (segment
  * length of the plan's first type) and re-applied without timing by
  * anim_set_schedule (for example in another process); CTAs per SM is 1, 2
@@ -368,6 +369,13 @@ ANIM_API int anim_tune_ik(anim_ctx *ctx, anim_plan *plan, int n_eff, const int32
  * schedule it was created under.  Synchronous; not capturable. */
 ANIM_API int anim_get_schedule(anim_ctx *ctx, const anim_plan *plan, int32_t *out5);
 ANIM_API int anim_set_schedule(anim_ctx *ctx, anim_plan *plan, const int32_t *in5);
+
+/* What of a plan runs on the chain-walk kernel in anim_evaluate_frame under
+ * the present schedule: *out_joints receives the number of its joints (0 if
+ * all run on the segmented kernel, the plan's total if none do),
+ * *out_lanes (nullable) the largest number of lanes a character of these
+ * types is walked by (0 without any). */
+ANIM_API int anim_plan_walk(anim_ctx *ctx, const anim_plan *plan, int64_t *out_joints, int32_t *out_lanes);
 
 /* Read and clear the device status word (synchronizes `stream`). */
 ANIM_API int anim_get_status(anim_ctx *ctx, void *stream, int *out_status);

@@ -825,6 +825,9 @@ struct Sched {
   int C = 1;  // characters per item
 };
 
+// The schedule's fourth value.
+enum { kWalkNever = 0, kWalkAlways = 1, kWalkByBatch = 2 };
+
 }  // namespace
 
 // ------------------------------------------------------------ ABI objects
@@ -862,6 +865,7 @@ struct anim_plan {
   // (d_queue[2..3])
   int n_slots_walk = 0;
   int walk_nbs = 0;
+  std::vector<char> on_walk;  // per ctx type id
   size_t walk_smem = 0;
   // frame with skinning: every type on the segmented CTA kernel (its own
   // range layout when the frame's layout gives some types to the walk kernel)
@@ -931,8 +935,7 @@ struct anim_ctx {
   int *d_status = nullptr;
   int version = 0;  // bumps when types/schedules change
   int ctas_per_sm = 2;            // resident persistent CTAs per SM the schedule is sized for
-  int use_walk = 1;               // frame: walkable types run on the chain-walk kernel (nonzero;
-                                  // two values from when it had two variants)
+  int use_walk = kWalkByBatch;    // frame: which walkable types run on the chain-walk kernel
   int adj_ctas = 0;               // adjoint: 0 = persistent kernel, k = one-item kernel sized for k CTAs per SM
   cudaStream_t side = nullptr;    // frame: the CTA kernel's stream when both kernels have work
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -1103,8 +1106,8 @@ std::vector<WorkItem> make_items(const anim_plan *P, const std::vector<int> &Cv)
   return items;
 }
 
-// Whether the plan's walkable types run on the chain-walk kernel under a
-// schedule that allows it.  The walk's time is its longest schedule's, S
+// Which types of a plan run on the chain-walk kernel (per type id): none, all
+// walkable ones, or all of them if the batch makes the walk pay.  The walk's time is its longest schedule's, S
 // steps whatever the batch, until its warps fill the chip; the segmented
 // kernel's is a short item's, then grows with the joints, and a joint costs
 // it more.  So the walk needs a batch, the larger the longer the schedule.
@@ -1119,8 +1122,9 @@ std::vector<WorkItem> make_items(const anim_plan *P, const std::vector<int> &Cv)
 //     33.7/32.7, 2.1 million 57.6/47.7.
 // 165 S^2 joints lie on or a little below where each pair meets.
 constexpr int64_t kWalkJointsPerStep2 = 165;
-bool walk_pays(const anim_ctx *ctx, const anim_plan *P) {
-  if (!ctx->use_walk) return false;
+std::vector<char> walk_types(const anim_ctx *ctx, const anim_plan *P, int mode) {
+  std::vector<char> on(ctx->types.size(), 0);
+  if (mode == kWalkNever) return on;
   int64_t joints = 0, S = 0;
   for (size_t u = 0; u < P->used.size(); ++u) {
     const TypeHost &T = *ctx->types[P->used[u]];
@@ -1128,7 +1132,9 @@ bool walk_pays(const anim_ctx *ctx, const anim_plan *P) {
     joints += (int64_t)T.n * (int64_t)P->by_type[u].size();
     S = std::max<int64_t>(S, T.ws.S);
   }
-  return joints >= kWalkJointsPerStep2 * S * S;
+  if (mode == kWalkByBatch && joints < kWalkJointsPerStep2 * S * S) return on;
+  for (int t : P->used) on[t] = ctx->types[t]->walk_ready();
+  return on;
 }
 
 // (Re)build the schedule-dependent parts of a plan: characters per item,
@@ -1141,15 +1147,14 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   for (auto *v : {&P->C_fwd, &P->C_frame, &P->C_layers}) v->assign(nt, 1);
   P->adj_unfit = -1;
   size_t smem_s = 0, smem_a = 0, smem_q = 0, smem_l = 0;
-  const bool walks = walk_pays(ctx, P);
-  auto on_walk = [&](const TypeHost &T) { return walks && T.walk_ready(); };
+  P->on_walk = walk_types(ctx, P, ctx->use_walk);
   std::vector<BatchType> all, adj, seg;  // every type, its adjoint view, the types off the walk kernel
   for (size_t u = 0; u < P->used.size(); ++u) {
     const TypeHost &T = *ctx->types[P->used[u]];
     const int64_t cnt = (int64_t)P->by_type[u].size();
     all.push_back({&T, cnt});
     adj.push_back({T.adj.get(), cnt});
-    if (!on_walk(T)) seg.push_back({&T, cnt});
+    if (!P->on_walk[P->used[u]]) seg.push_back({&T, cnt});
   }
   const int ctas = ctx->sm_count * ctx->ctas_per_sm;
   const int t_fwd = item_target(ctx, all, ctas, 2, false), t_frame = item_target(ctx, seg, ctas, 2, true),
@@ -1187,17 +1192,15 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   // plain frame: walkable types (chain-walk kernel, 32 / P characters per
   // item) take the first item regions, the others ((q, t) items) follow
   std::vector<int32_t> cap(P->C_frame);
-  std::vector<char> walk_t(nt, 0);
   int wcmax = 0;
   size_t smem_f = 0;
   P->walk_nbs = 0;
   for (int t : P->used) {
     const TypeHost &T = *ctx->types[t];
-    if (!on_walk(T)) {
+    if (!P->on_walk[t]) {
       smem_f = std::max(smem_f, scan_qt_smem_bytes(T.n, T.seg.nseg, P->C_frame[t]));
       continue;
     }
-    walk_t[t] = 1;
     cap[t] = 32 / T.ws.P;
     wcmax = std::max(wcmax, cap[t]);
     P->walk_nbs = std::max(P->walk_nbs, T.ws.nbs);
@@ -1211,7 +1214,7 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   for (int pass = 0; pass < 2; ++pass) {
     for (size_t u = 0; u < P->used.size(); ++u) {
       const int t = P->used[u];
-      if (walk_t[t] != (pass == 0)) continue;
+      if (P->on_walk[t] != (pass == 0)) continue;
       const int cnt = (int)P->by_type[u].size(), C = cap[t], nk = ctx->types[t]->n_keys;
       const int rc = pass == 0 ? kRangeCharsMax : kRangeChars;
       for (int k = 0; k < cnt; k += rc) {
@@ -2275,12 +2278,15 @@ static int apply_choice(anim_ctx *ctx, const anim_plan *P, int seg_len, int cps,
 // context's settings.
 extern "C++" {  // a template inside the ABI's extern "C" block
 template <class F>
-static void for_each_candidate(const anim_ctx *ctx, int which, F &&f) {
+static void for_each_candidate(const anim_ctx *ctx, const anim_plan *plan, int which, F &&f) {
   const int segs[] = {4, 8, 16, 32}, cpss[] = {1, 2, 3}, jpis[] = {256, 512, 1024, 2048, 4096};
   const int adjs[] = {0, 4, 6, 7, 8};
-  const int walk_lo = which == 0 ? 0 : ctx->use_walk, walk_hi = which == 0 ? 2 : ctx->use_walk;
+  const int walks[] = {kWalkByBatch, kWalkNever, kWalkAlways}, walk_keep = ctx->use_walk;
   const int adj_keep = ctx->adj_ctas;
-  for (int walk = walk_lo; walk <= walk_hi; walk += 2)  // 1 and 2 run the same kernel
+  std::set<std::vector<char>> seen;  // by batch first: it is the better of equals for the context's other plans
+  for (int w = 0; w < (which == 0 ? 3 : 1); ++w) {
+    const int walk = which == 0 ? walks[w] : walk_keep;
+    if (!seen.insert(walk_types(ctx, plan, walk)).second) continue;
     for (int adj : adjs)
       for (int seg : segs)
         for (int cps : cpss)
@@ -2292,6 +2298,7 @@ static void for_each_candidate(const anim_ctx *ctx, int which, F &&f) {
             if (which == 2 && adj_c > 0 && cps != 2) continue;  // CTAs per SM of the persistent kernels: unused
             f(seg, cps, jpi, walk, adj_c);
           }
+  }
 }
 }  // extern "C++"
 
@@ -2409,7 +2416,7 @@ int anim_tune(anim_ctx *ctx, anim_plan *plan, int which) {
     return ok;
   };
   anim_ctx::TuneChoice best{0, 0, 0, 0, 0, 1e30f};
-  for_each_candidate(ctx, which, [&](int seg, int cps, int jpi, int walk, int adj_c) {
+  for_each_candidate(ctx, plan, which, [&](int seg, int cps, int jpi, int walk, int adj_c) {
     if (apply_choice(ctx, plan, seg, cps, jpi, walk, adj_c) != ANIM_OK) return;  // e.g. does not fit
     bool ok = true;
     for (int w = 0; w < 2 && ok; ++w) ok = run_once(ts) == ANIM_OK;  // outside capture: attributes, side stream
@@ -2481,7 +2488,7 @@ int anim_tune_ik(anim_ctx *ctx, anim_plan *plan, int n_eff, const int32_t *effec
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   anim_ctx::TuneChoice best{0, 0, 0, 0, 0, 1e30f};
-  for_each_candidate(ctx, 2, [&](int seg, int cps, int jpi, int walk, int adj_c) {
+  for_each_candidate(ctx, plan, 2, [&](int seg, int cps, int jpi, int walk, int adj_c) {
     if (apply_choice(ctx, plan, seg, cps, jpi, walk, adj_c) != ANIM_OK) return;  // e.g. does not fit
     anim_ik *ik = nullptr;
     if (anim_ik_create(ctx, plan, n_eff, effectors, &ik) != ANIM_OK) return;  // a view does not fit
@@ -2519,6 +2526,23 @@ int anim_get_schedule(anim_ctx *ctx, const anim_plan *plan, int32_t *out5) {
   out5[2] = ctx->joints_per_item;
   out5[3] = ctx->use_walk;
   out5[4] = ctx->adj_ctas;
+  return ANIM_OK;
+}
+
+int anim_plan_walk(anim_ctx *ctx, const anim_plan *plan, int64_t *out_joints, int32_t *out_lanes) {
+  int rc = check_plan(ctx, plan);
+  if (rc) return rc;
+  if (!out_joints) return fail(ctx, ANIM_EINVAL, "out_joints is NULL");
+  int64_t joints = 0;
+  int lanes = 0;
+  for (size_t u = 0; u < plan->used.size(); ++u) {
+    if (!plan->on_walk[plan->used[u]]) continue;
+    const TypeHost &T = *ctx->types[plan->used[u]];
+    joints += (int64_t)T.n * (int64_t)plan->by_type[u].size();
+    lanes = std::max(lanes, T.ws.P);
+  }
+  *out_joints = joints;
+  if (out_lanes) *out_lanes = lanes;
   return ANIM_OK;
 }
 
