@@ -299,10 +299,13 @@ struct RasterArgs {
   uint32_t *rgba;                 // nullable
   int width, height, cols;
   float spacing, ox, oy, scale;
-  int stage_verts;                // set by launch_raster: vertices the shared-memory stage holds
+  int stage_verts;                // vertices the shared-memory stage holds, at most kRasterStageVerts
 };
-// max_verts: the largest vertex count among the characters' types.
-cudaError_t launch_raster(const RasterArgs &a, int n_chars, int max_verts, cudaStream_t s);
+// Vertices of a character staged in shared memory, 12 bytes each: 48 KB and
+// the warps' triangles keep three CTAs on an SM.
+constexpr int kRasterStageVerts = 4096;
+// all_staged: no character has more than a.stage_verts vertices.
+cudaError_t launch_raster(const RasterArgs &a, int n_chars, bool all_staged, cudaStream_t s);
 
 // Setup kernels.
 cudaError_t launch_prepare_keys(float4 *keys, int n_clips, int n_keys, int n, cudaStream_t s);

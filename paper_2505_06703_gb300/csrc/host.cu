@@ -1551,9 +1551,15 @@ int anim_raster(anim_ctx *ctx, const anim_plan *plan, const float *d_verts, cons
   a.ox = params->ox;
   a.oy = params->oy;
   a.scale = params->scale;
-  int max_verts = 0;
-  for (int t : plan->used) max_verts = std::max(max_verts, ctx->types[t]->n_verts);
-  CK(launch_raster(a, (int)plan->n_chars, max_verts, (cudaStream_t)stream));
+  bool all_staged = true;
+  for (int t : plan->used) {
+    const int nv = ctx->types[t]->n_verts;
+    if (nv <= kRasterStageVerts)
+      a.stage_verts = std::max(a.stage_verts, nv);
+    else
+      all_staged = false;
+  }
+  CK(launch_raster(a, (int)plan->n_chars, all_staged, (cudaStream_t)stream));
   return ANIM_OK;
 }
 

@@ -54,9 +54,12 @@ __device__ __forceinline__ void put_pixel(unsigned long long *at, float e0, floa
   atomicMin(at, ((unsigned long long)__float_as_uint(d) << 32) | id);
 }
 
+// Depth of a vertex.
+__device__ __forceinline__ float depth_of(float z) { return (2.f - z) * 0.25f; }
+
 // One triangle in 64-bit arithmetic straight from the vertices: whatever
 // the 32-bit path below does not take (far off-screen or non-finite
-// positions, triangles of 64 pixels and more, meshes too large to stage).
+// positions, triangles of 64 pixels and more).
 __device__ __noinline__ void raster_tri_wide(const RasterArgs &a, const float *vb, const int32_t *face, int c,
                                              unsigned int id) {
   long long X[3], Y[3];
@@ -66,7 +69,7 @@ __device__ __noinline__ void raster_tri_wide(const RasterArgs &a, const float *v
     const float2 p = to_screen(a, c, __ldcg(v), __ldcg(v + 1));
     X[k] = llroundf(p.x);
     Y[k] = llroundf(p.y);
-    D[k] = (2.f - __ldcg(v + 2)) * 0.25f;
+    D[k] = depth_of(__ldcg(v + 2));
   }
   long long area = (X[1] - X[0]) * (Y[2] - Y[0]) - (Y[1] - Y[0]) * (X[2] - X[0]);
   if (area == 0) return;
@@ -111,6 +114,11 @@ constexpr int kFar = (int)0x80000000;
 __device__ __forceinline__ int snap_32(float v) {
   const float s = roundf(v);  // halves away from zero, as llroundf
   return fabsf(s) < 1073741824.f ? (int)s : kFar;
+}
+
+__device__ __forceinline__ int2 snapped_corner(const RasterArgs &a, int c, const float *v) {
+  const float2 s = to_screen(a, c, __ldcg(v), __ldcg(v + 1));
+  return make_int2(snap_32(s.x), snap_32(s.y));
 }
 
 // The sides of the image a snapped position lies past, so that no pixel
@@ -197,6 +205,11 @@ __device__ __forceinline__ void test_pixel(const RasterArgs &a, const WarpTris &
 // edges, 176 with a row per lane, 112 as it is (83.8 M warp instructions at
 // 75 % issue; the vertices' 147 MB take 22 us).  A 5-CTA build spills: 116;
 // three CTAs per SM: 122.
+// ALL_STAGED: every mesh fits the stage.  Otherwise the characters of the
+// larger ones snap each triangle's corners as they come to it: 1,500 of 4,500
+// vertices and 4,096 faces, 64 columns, take 177 us (686 with a triangle per
+// lane in 64 bits, 2,582 with these meshes left to raster_tri_wide).
+template <bool ALL_STAGED>
 __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_tris(const __grid_constant__ RasterArgs a) {
   extern __shared__ int2 sxy[];
   __shared__ WarpTris tris[kRasterThreads / 32];
@@ -208,7 +221,7 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_tris(const __grid_
   const int nf = T.n_faces, nv = nf > 0 ? T.n_verts : 0;
   const float *vb = a.verts + a.vert_off[c] * 6;
   float *sd = reinterpret_cast<float *>(sxy + a.stage_verts);
-  const bool staged = nv <= a.stage_verts;
+  const bool staged = ALL_STAGED || nv <= a.stage_verts;
   unsigned code = staged ? 15u : 0u;  // no vertices: past every side
   if (staged) {
     if ((reinterpret_cast<uintptr_t>(vb) & 7u) == 0) {
@@ -220,7 +233,7 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_tris(const __grid_
         const float2 s = to_screen(a, c, p.x, p.y);
         const int2 xy = make_int2(snap_32(s.x), snap_32(s.y));
         sxy[v] = xy;
-        sd[v] = (2.f - z) * 0.25f;
+        sd[v] = depth_of(z);
         code &= outside(a, xy.x, xy.y);
       }
     } else {
@@ -228,7 +241,7 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_tris(const __grid_
         const float2 s = to_screen(a, c, __ldcg(vb + 6 * v), __ldcg(vb + 6 * v + 1));
         const int2 xy = make_int2(snap_32(s.x), snap_32(s.y));
         sxy[v] = xy;
-        sd[v] = (2.f - __ldcg(vb + 6 * v + 2)) * 0.25f;
+        sd[v] = depth_of(__ldcg(vb + 6 * v + 2));
         code &= outside(a, xy.x, xy.y);
       }
     }
@@ -260,10 +273,12 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_tris(const __grid_
       n1 = __ldg(faces + 3 * (f + kRasterThreads) + 1);
       n2 = __ldg(faces + 3 * (f + kRasterThreads) + 2);
     }
-    bool wide = f < nf && !staged;
+    bool wide = false;
     int lines = 0, X0 = 0, Y0 = 0, X1 = 0, Y1 = 0, X2 = 0, Y2 = 0, px0 = 0, pw = 0, py0 = 0, ph = 0, area = 0;
-    if (f < nf && staged) {
-      const int2 p0 = sxy[i0], p1 = sxy[i1], p2 = sxy[i2];
+    if (f < nf) {
+      const int2 p0 = staged ? sxy[i0] : snapped_corner(a, c, vb + 6 * (long long)i0),
+                 p1 = staged ? sxy[i1] : snapped_corner(a, c, vb + 6 * (long long)i1),
+                 p2 = staged ? sxy[i2] : snapped_corner(a, c, vb + 6 * (long long)i2);
       X0 = p0.x, Y0 = p0.y, X1 = p1.x, Y1 = p1.y, X2 = p2.x, Y2 = p2.y;
       const int xmin = min(X0, min(X1, X2)), xmax = max(X0, max(X1, X2));
       const int ymin = min(Y0, min(Y1, Y2)), ymax = max(Y0, max(Y1, Y2));
@@ -314,7 +329,10 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_tris(const __grid_
       W.r[lane] = make_int4(r0, r1, r2, py0 * a.width + px0);  // below 2^28
       W.a[lane] = make_int4(u0, u1, u2, f | (b0 | b1 << 1 | b2 << 2 | (cols ? 8 : 0)) << 12);
       W.b[lane] = make_int4(s0, s1, s2, __float_as_int(1.f / (float)area));
-      W.D[lane] = make_float4(sd[i0], sd[i1], sd[i2], 0.f);
+      W.D[lane] = staged ? make_float4(sd[i0], sd[i1], sd[i2], 0.f)
+                         : make_float4(depth_of(__ldcg(vb + 6 * (long long)i0 + 2)),
+                                       depth_of(__ldcg(vb + 6 * (long long)i1 + 2)),
+                                       depth_of(__ldcg(vb + 6 * (long long)i2 + 2)), 0.f);
     }
     const Bracket k0 = bracket_of(s0), k1 = bracket_of(s1), k2 = bracket_of(s2);
     const float len = (float)max(pw, ph);
@@ -389,11 +407,6 @@ __global__ void k_raster_resolve(const RasterArgs a) {
 
 }  // namespace
 
-// Vertices of a character staged in shared memory, 12 bytes each: 48 KB and
-// the warps' triangles keep three CTAs on an SM.  Larger meshes take the wide
-// path.
-constexpr int kRasterStageVerts = 4096;
-
 template <class... Args>
 static cudaError_t launch_chained(void (*k)(Args...), unsigned grid, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t lc = {};
@@ -409,19 +422,18 @@ static cudaError_t launch_chained(void (*k)(Args...), unsigned grid, size_t smem
   return cudaLaunchKernelEx(&lc, k, args...);
 }
 
-cudaError_t launch_raster(const RasterArgs &args, int n_chars, int max_verts, cudaStream_t st) {
-  const long long n = (long long)args.width * args.height;
+cudaError_t launch_raster(const RasterArgs &a, int n_chars, bool all_staged, cudaStream_t st) {
+  const long long n = (long long)a.width * a.height;
   const unsigned blocks = (unsigned)std::max(1ll, std::min((n + 255) / 256, 4096ll));
-  cudaError_t e = launch_chained(k_raster_clear, blocks, 0, st, args.vis, n);
+  cudaError_t e = launch_chained(k_raster_clear, blocks, 0, st, a.vis, n);
   if (e != cudaSuccess) return e;
-  RasterArgs a = args;
-  a.stage_verts = std::min(max_verts, kRasterStageVerts);
   if (n_chars > 0) {
-    static SmemLimit lim;
+    static SmemLimit lims[2];
+    const auto kernel = all_staged ? k_raster_tris<true> : k_raster_tris<false>;
     const size_t smem = 12 * (size_t)a.stage_verts;
-    e = ensure_smem_limit((const void *)k_raster_tris, lim, smem);
+    e = ensure_smem_limit((const void *)kernel, lims[all_staged], smem);
     if (e != cudaSuccess) return e;
-    e = launch_chained(k_raster_tris, (unsigned)n_chars, smem, st, a);
+    e = launch_chained(kernel, (unsigned)n_chars, smem, st, a);
     if (e != cudaSuccess) return e;
   }
   return launch_chained(k_raster_resolve, blocks, 0, st, a);
