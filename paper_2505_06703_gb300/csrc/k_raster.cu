@@ -59,9 +59,14 @@ __device__ __forceinline__ float depth_of(float z) { return (2.f - z) * 0.25f; }
 
 // One triangle in 64-bit arithmetic straight from the vertices: whatever
 // the 32-bit path below does not take (far off-screen or non-finite
-// positions, triangles of 64 pixels and more).
+// positions, triangles of 64 pixels and more).  The warp takes it together,
+// a pixel per lane along the longer side of its box: such triangles have up
+// to tens of thousands of pixels, and a lane walking one alone is what the
+// launch then waits for (1920x1080, 142 pixels per unit, 30 characters of 308
+// faces: 2,311 us with every triangle on a lane of its own, 2,785 with the
+// small ones taken by the warp first, 969 as it is).
 __device__ __noinline__ void raster_tri_wide(const RasterArgs &a, const float *vb, const int32_t *face, int c,
-                                             unsigned int id) {
+                                             unsigned int id, int lane) {
   long long X[3], Y[3];
   float D[3];
   for (int k = 0; k < 3; ++k) {
@@ -89,9 +94,13 @@ __device__ __noinline__ void raster_tri_wide(const RasterArgs &a, const float *v
   const long long ymin = min(Y[0], min(Y[1], Y[2])), ymax = max(Y[0], max(Y[1], Y[2]));
   const long long px0 = max(0ll, (xmin - 128 + 255) >> 8), px1 = min((long long)a.width - 1, (xmax - 128) >> 8);
   const long long py0 = max(0ll, (ymin - 128 + 255) >> 8), py1 = min((long long)a.height - 1, (ymax - 128) >> 8);
+  if (px1 < px0 || py1 < py0) return;
   const float inv_area = 1.f / (float)area;
-  for (long long py = py0; py <= py1; ++py) {
-    for (long long px = px0; px <= px1; ++px) {
+  const bool cols = px1 - px0 < py1 - py0;
+  const int len = (int)(cols ? py1 - py0 : px1 - px0), lines = (int)(cols ? px1 - px0 : py1 - py0);
+  for (int line = 0; line <= lines; ++line) {
+    for (int at = lane; at <= len; at += 32) {
+      const long long px = px0 + (cols ? line : at), py = py0 + (cols ? at : line);
       const long long cx = px * 256 + 128, cy = py * 256 + 128;
       long long e[3];
       bool inside = true;
@@ -367,8 +376,11 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_tris(const __grid_
   }
   if (any_wide == 0) return;
   __syncwarp();
-  for (f = tid; f - lane < nf; f += kRasterThreads)  // the warp's own faces again
-    if (wide_faces[f >> 5] >> lane & 1u) raster_tri_wide(a, vb, faces + 3 * f, c, cid + (unsigned)f);
+  for (f = tid - lane; f < nf; f += kRasterThreads)  // the warp's own faces again
+    for (unsigned w = wide_faces[f >> 5]; w; w &= w - 1u) {
+      const int g = f + __ffs(w) - 1;
+      raster_tri_wide(a, vb, faces + 3 * g, c, cid + (unsigned)g, lane);
+    }
 }
 
 __global__ void k_raster_resolve(const RasterArgs a) {
