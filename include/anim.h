@@ -354,8 +354,8 @@ ANIM_API int anim_tune_ik(anim_ctx *ctx, anim_plan *plan, int n_eff, const int32
 /* The schedule the autotuner picked, as 5 integers: segment length, resident
  * CTAs per SM, work-item size in joints (an upper bound: a batch that does
  * not fill the chip at that size takes smaller items), chain-walk kernel for
- * the frame (0: never, 1: for every walkable type, 2, the default: for
- * walkable types in batches large enough that it is the faster kernel;
+ * the frame (0: never, 1: for every walkable type, 2, the default: for the
+ * walkable types whose batch is large enough that it is the faster kernel;
  * anim_plan_walk tells), adjoint kernel (0: persistent, k = 1..8: one work item per CTA,
  * items sized so k CTAs share an SM) -- read with anim_get_schedule (segment
  * length of the plan's first type) and re-applied without timing by

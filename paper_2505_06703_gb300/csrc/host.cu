@@ -1107,33 +1107,54 @@ std::vector<WorkItem> make_items(const anim_plan *P, const std::vector<int> &Cv)
 }
 
 // Which types of a plan run on the chain-walk kernel (per type id): none, all
-// walkable ones, or all of them if the batch makes the walk pay.  The walk's time is its longest schedule's, S
-// steps whatever the batch, until its warps fill the chip; the segmented
-// kernel's is a short item's, then grows with the joints, and a joint costs
-// it more.  So the walk needs a batch, the larger the longer the schedule.
-// Measured, us on the segmented kernel / the walk:
+// walkable ones, or those that the batch makes it pay for.  The walk's time is
+// its longest schedule's, S steps whatever the batch, until its warps fill
+// the chip; the segmented kernel's is a short item's, then grows with the
+// joints, and a joint costs it more.  So the walk needs a batch, the larger
+// the longer the schedule.  Measured, us on the segmented kernel / the walk:
 //   67 joints, S about 16: 41 thousand joints 10.7/10.8, 67 thousand
 //     11.6/11.5, 134 thousand 14.4/12.5;
-//   ragged 200, 126, 53 joints, S about 40: 126 thousand 14.0/20.9, 250
-//     thousand 20.0/22.5, 500 thousand 30.4/27.9;
+//   ragged 200, 126, 53 joints, S about 50: 250 thousand 20.0/22.8, 380
+//     thousand 23.9/24.5, 505 thousand 30.4/28.2;
 //   300 joints, S about 64: 12 thousand 11.5/23.6, 300 thousand 20.4/28.0,
 //     600 thousand 33.0/32.7, 1.2 million 56.9/42.2;
 //   512-joint bipeds, S about 70: 0.5 million 20.8/27.6, 1.0 million
 //     33.7/32.7, 2.1 million 57.6/47.7.
-// 165 S^2 joints lie on or a little below where each pair meets.
+// They meet at about 140 to 200 S^2 joints; the line is drawn at 165.
+// All walkable types go if their joints reach that line for the longest
+// schedule among them.  If not, a rare type with a long schedule must not
+// keep a crowd off the walk: the types of the shortest schedules that reach
+// their own line go alone.  The others then run beside them on a second
+// stream, which costs a few us and takes SMs from the walk, so only where
+// the walk keeps 400 thousand joints and at least 8 of 9 of the plan's.
+// 4,096 bipeds and a dragon with 1 / 300 / 1,000 chains of 120 joints: 67.5 /
+// 67.7 / 68.7 us all segmented, 65.3 / 73.4 / 76.1 all walked, 46.1 / 46.5 /
+// 51.8 with the chains left segmented.  Smaller batches and shares turn it:
+// trees of 128 joints beside trees of 300, 200 and 25 thousand joints 17.9
+// all segmented, 20.3 apart; 400 and 100 thousand 27.6 and 29.2; but 400 and
+// 25 thousand 23.9 and 23.3, 800 and 100 thousand 37.4 and 35.0.
 constexpr int64_t kWalkJointsPerStep2 = 165;
+constexpr int64_t kWalkAloneJoints = 400000, kWalkAloneShare = 8;
 std::vector<char> walk_types(const anim_ctx *ctx, const anim_plan *P, int mode) {
   std::vector<char> on(ctx->types.size(), 0);
   if (mode == kWalkNever) return on;
-  int64_t joints = 0, S = 0;
+  std::vector<std::pair<int64_t, int64_t>> steps;  // (S, joints) of each walkable type
   for (size_t u = 0; u < P->used.size(); ++u) {
     const TypeHost &T = *ctx->types[P->used[u]];
-    if (!T.walk_ready()) continue;
-    joints += (int64_t)T.n * (int64_t)P->by_type[u].size();
-    S = std::max<int64_t>(S, T.ws.S);
+    if (T.walk_ready()) steps.push_back({T.ws.S, (int64_t)T.n * (int64_t)P->by_type[u].size()});
   }
-  if (mode == kWalkByBatch && joints < kWalkJointsPerStep2 * S * S) return on;
-  for (int t : P->used) on[t] = ctx->types[t]->walk_ready();
+  std::sort(steps.begin(), steps.end());
+  int64_t most = mode == kWalkAlways ? INT64_MAX : 0, joints = 0;
+  if (mode == kWalkByBatch)
+    for (size_t i = 0; i < steps.size(); ++i) {
+      const int64_t S = steps[i].first;
+      joints += steps[i].second;
+      if (i + 1 < steps.size() && (steps[i + 1].first == S || joints < kWalkAloneJoints ||
+                                   joints < kWalkAloneShare * (P->total - joints)))
+        continue;
+      if (joints >= kWalkJointsPerStep2 * S * S) most = S;
+    }
+  for (int t : P->used) on[t] = ctx->types[t]->walk_ready() && ctx->types[t]->ws.S <= most;
   return on;
 }
 

@@ -132,3 +132,21 @@ def test_given_inverse_binds(bind):
     out = ctx.evaluate_frame(plan, *_inputs(w))
     for ty, e in _gpu.per_type_maxabs(out.cpu().numpy(), ref, w).items():
         assert e <= scale * _gpu.tol_for_depth(w["types"][ty]["depth"]), (ty, e)
+
+
+@pytest.mark.parametrize("small,props,walked", [(6200, 2, (0,)), (6200, 400, ()), (3000, 2, ()), (6200, 0, (0,))])
+def test_rare_long_type_beside_a_crowd(small, props, walked):
+    """By batch: a 67-joint crowd large enough for the walk keeps it beside a few 150-joint chains, whose own line
+    lies at millions of joints; not beside chains that are a seventh of the joints, nor below 400 thousand."""
+    rng = np.random.default_rng(small + props)
+    tree = synth.relabel_dfs(synth.random_tree(67, 14, rng, spine=14), rng)[0]
+    w = _workload([tree, synth.chain(150)], small + props, rng)
+    w["char_type"][:] = 0
+    w["char_type"][rng.permutation(small + props)[:props]] = 1
+    ctx, plan = _gpu.setup(w)
+    assert ctx.get_schedule(plan)[3] == 2
+    assert ctx.plan_walk(plan)[0] == _joints(w, walked)
+    out = ctx.evaluate_frame(plan, *_inputs(w))
+    _gpu.assert_skin_close(out.cpu().numpy(), oracle.frame(w), w)
+    ctx.set_schedule(plan, [16, 2, 2048, 1, 0])
+    assert ctx.plan_walk(plan)[0] == plan.total
