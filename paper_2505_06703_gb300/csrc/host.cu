@@ -1808,16 +1808,28 @@ int anim_evaluate_frame(anim_ctx *ctx, const anim_plan *plan, const float *d_tim
 // kHostPartMinChars characters.  The copy-out is the long pole (5 times the
 // frame at the link's 192 GB/s) and can start when the first range is done,
 // so ranges grow: range i ends at the share (i / kHostParts)^2 of the joints,
-// and each range's copy covers the next one's frame.
-// 576 -> 561 us for 4,097 bipeds' 100.7 MB (four equal ranges before).
+// and each range's copy covers the next one's frame -- if it is as long: a
+// frame of few characters still takes 10 us for the work queue and the
+// launches and the time of its longest type, S / 3 us on the chain walk, n /
+// 200 on the segmented kernel, and the link moves 4,000 joints per us, so no
+// range has fewer joints than that.  Measured, us with four equal ranges /
+// growing ones without that floor / as it is: 2,000 characters of 21 joints
+// 55/61/38, of 67 joints 71/77/67, of the five mixed types 212/218/213; 1,100
+// bipeds and a dragon 186/176/174, 4,096 of them (100.7 MB, on the walk)
+// 572/567/567.
 constexpr int kHostParts = 4;
 constexpr int64_t kHostPartMinChars = 1024;
 
 static int make_host_parts(anim_ctx *ctx, anim_plan *plan) {
   const int64_t N = plan->n_chars, total = plan->total;
+  int64_t least = 0;
+  for (int t : plan->used) {
+    const TypeHost &T = *ctx->types[t];
+    least = std::max<int64_t>(least, 40000 + (plan->on_walk[t] ? 4000 * T.ws.S / 3 : 20 * T.n));
+  }
   std::vector<int64_t> cut = {0};
   for (int k = 1; k < kHostParts; ++k) {
-    const int64_t target = total * k * k / (kHostParts * kHostParts);
+    const int64_t target = std::max(total * k * k / (kHostParts * kHostParts), k * least);
     int64_t c = cut.back();
     while (c < N && plan->row_off[c] < target) ++c;
     if (c > cut.back() && c < N) cut.push_back(c);
