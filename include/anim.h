@@ -178,6 +178,9 @@ ANIM_API int anim_evaluate_frame(anim_ctx *ctx, const anim_plan *plan, const flo
  * copied in, the frame runs as in anim_evaluate_frame, and the skin matrices
  * are copied back into h_skin (host [total][12] float), all in order on
  * `stream`; the output is complete once `stream` has synchronized.
+ * The matrices are anim_evaluate_frame's bit for bit, but for pure chains of
+ * more than 1,024 joints: how many of those share a work item, and by that
+ * the order of their products, depends on the range they are evaluated in.
  * Page-locked buffers (cudaMallocHost, cudaHostRegister) make the copies
  * asynchronous; pageable ones work through the driver's staging.  A plan of
  * at least 1,024 characters is evaluated in up to 4 contiguous ranges of

@@ -833,6 +833,7 @@ enum { kWalkNever = 0, kWalkAlways = 1, kWalkByBatch = 2 };
 // ------------------------------------------------------------ ABI objects
 struct anim_plan {
   anim_ctx *ctx = nullptr;
+  const anim_plan *whole = nullptr;  // of a range of the host-buffer frame: the plan it is cut from
   int64_t n_chars = 0;
   std::vector<int32_t> char_type;
   std::vector<int64_t> row_off;
@@ -1168,7 +1169,9 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   for (auto *v : {&P->C_fwd, &P->C_frame, &P->C_layers}) v->assign(nt, 1);
   P->adj_unfit = -1;
   size_t smem_s = 0, smem_a = 0, smem_q = 0, smem_l = 0;
-  P->on_walk = walk_types(ctx, P, ctx->use_walk);
+  // a range of the host-buffer frame runs on the kernels that its whole plan
+  // runs on: they round differently
+  P->on_walk = walk_types(ctx, P->whole ? P->whole : P, ctx->use_walk);
   std::vector<BatchType> all, adj, seg;  // every type, its adjoint view, the types off the walk kernel
   for (size_t u = 0; u < P->used.size(); ++u) {
     const TypeHost &T = *ctx->types[P->used[u]];
@@ -1592,7 +1595,8 @@ int anim_plan_vertex_offsets(anim_ctx *ctx, const anim_plan *plan, int64_t *out)
   return ANIM_OK;
 }
 
-int anim_plan_create(anim_ctx *ctx, int64_t n_chars, const int32_t *char_type, anim_plan **out) {
+static int plan_create(anim_ctx *ctx, int64_t n_chars, const int32_t *char_type, const anim_plan *whole,
+                       anim_plan **out) {
   if (!ctx) return ANIM_EINVAL;
   if (!out || n_chars < 0 || (n_chars > 0 && !char_type)) return fail(ctx, ANIM_EINVAL, "bad plan arguments");
   if (n_chars > (int64_t)kRangeChars * (kMaxRanges - kMaxTypes))
@@ -1606,6 +1610,7 @@ int anim_plan_create(anim_ctx *ctx, int64_t n_chars, const int32_t *char_type, a
   CK(cudaSetDevice(ctx->device));
   std::unique_ptr<anim_plan> P(new anim_plan());
   P->ctx = ctx;
+  P->whole = whole;
   P->n_chars = n_chars;
   P->char_type.assign(char_type, char_type + n_chars);
   P->row_off.resize(n_chars + 1);
@@ -1644,6 +1649,10 @@ int anim_plan_create(anim_ctx *ctx, int64_t n_chars, const int32_t *char_type, a
   ctx->plans.insert(P.get());
   *out = P.release();
   return ANIM_OK;
+}
+
+int anim_plan_create(anim_ctx *ctx, int64_t n_chars, const int32_t *char_type, anim_plan **out) {
+  return plan_create(ctx, n_chars, char_type, nullptr, out);
 }
 
 int anim_plan_destroy(anim_ctx *ctx, anim_plan *plan) {
@@ -1838,7 +1847,7 @@ static int make_host_parts(anim_ctx *ctx, anim_plan *plan) {
   std::vector<anim_plan *> parts;
   for (size_t i = 0; i + 1 < cut.size(); ++i) {
     anim_plan *p = nullptr;
-    const int rc = anim_plan_create(ctx, cut[i + 1] - cut[i], plan->char_type.data() + cut[i], &p);
+    const int rc = plan_create(ctx, cut[i + 1] - cut[i], plan->char_type.data() + cut[i], plan, &p);
     if (rc != ANIM_OK) {
       for (anim_plan *q : parts) anim_plan_destroy(ctx, q);
       return rc;

@@ -150,3 +150,28 @@ def test_rare_long_type_beside_a_crowd(small, props, walked):
     _gpu.assert_skin_close(out.cpu().numpy(), oracle.frame(w), w)
     ctx.set_schedule(plan, [16, 2, 2048, 1, 0])
     assert ctx.plan_walk(plan)[0] == plan.total
+
+
+@pytest.mark.parametrize("chars,dragons", [(1500, 0), (4000, 3)])
+def test_host_frame_runs_on_the_device_frames_kernels(chars, dragons):
+    """The ranges of a host-buffer frame are below the walk's line where the whole batch is above it: they follow the
+    whole batch, so both entry points give the same bits."""
+    import torch
+    rng = np.random.default_rng(chars)
+    tree = synth.relabel_dfs(synth.random_tree(67, 14, rng, spine=14), rng)[0]
+    w = _workload([tree, synth.chain(600)], chars, rng)
+    w["char_type"][:] = 0
+    w["char_type"][rng.permutation(chars)[:dragons]] = 1
+    ctx, plan = _gpu.setup(w)
+    assert ctx.plan_walk(plan)[0] == 67 * (chars - dragons)
+    ref = ctx.evaluate_frame(plan, *_inputs(w)).cpu()
+    host = [torch.as_tensor(w[k]).pin_memory() for k in ("time", "weight")]
+    for _ in range(2):
+        out = ctx.evaluate_frame_host(plan, *host)
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
+    ctx.set_schedule(plan, [16, 2, 2048, 0, 0])  # the ranges follow a new schedule too
+    ref = ctx.evaluate_frame(plan, *_inputs(w)).cpu()
+    out = ctx.evaluate_frame_host(plan, *host)
+    torch.cuda.synchronize()
+    assert torch.equal(out, ref)
