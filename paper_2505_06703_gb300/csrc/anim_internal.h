@@ -64,8 +64,10 @@ struct TypeDev {
   // Skinned mesh (linear blend skinning after the bind product): 3 planes of
   // n_verts float4, (px py pz nx), (ny nz w0 w1), (w2 w3 bones01 bones23)
   // with the bone ids as 16-bit pairs in the last two words' bits; planes, so
-  // that a warp's loads are contiguous.
+  // that a warp's loads are contiguous.  mesh_zeros: some vertex has a zero
+  // first weight.
   int n_verts;
+  int mesh_zeros;
   int n_faces;
   const float4 *mesh;
   const int32_t *faces;      // [n_faces][3] vertex indices (raster)

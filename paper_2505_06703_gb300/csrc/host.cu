@@ -469,6 +469,7 @@ struct TypeHost {
   float4 *d_add = nullptr;      // additive layer keys [n_keys][n][2]
   float4 *d_mesh = nullptr;     // skinned mesh, 3 planes of n_verts float4
   int n_verts = 0;
+  bool mesh_zeros = false;      // a record with a zero first weight (pack_influences)
   int32_t *d_faces = nullptr;   // [n_faces][3]
   int n_faces = 0;
   float4 *d_wkeys = nullptr;    // schedule-ordered key records, inverse binds folded in
@@ -586,6 +587,7 @@ struct TypeHost {
     dev.wk_keys = d_wkeys;
     dev.wk_u = d_wu;
     dev.n_verts = n_verts;
+    dev.mesh_zeros = mesh_zeros;
     dev.mesh = d_mesh;
     dev.n_faces = n_faces;
     dev.faces = d_faces;
@@ -1468,6 +1470,37 @@ int anim_upload_additive(anim_ctx *ctx, int32_t type_id, int n_keys, float rate_
 
 static int check_plan(anim_ctx *ctx, const anim_plan *plan);
 
+// The influences of a mesh record.  Zero-weight slots are skipped: each takes
+// half of the weight, and the bone, of the slot that has the most, so that
+// the kernel need not test (a branch per slot cost it 5 of 113 us) and no
+// unused bone's pose, be it non-finite, enters the sum.  Where there is no
+// weight to halve (all zero, or so small that a half is not exact) the slots
+// keep their weights, the zero ones first: a zero first weight makes the
+// kernel test the vertex's slots.
+static void pack_influences(const float *weights, const int32_t *bones, float *w, int32_t *b) {
+  std::copy(weights, weights + 4, w);
+  std::copy(bones, bones + 4, b);
+  for (int k = 0; k < 4; ++k) {
+    if (w[k] != 0.f) continue;
+    int m = 0;
+    for (int i = 1; i < 4; ++i)
+      if (std::fabs(w[i]) > std::fabs(w[m])) m = i;
+    const float half = w[m] * 0.5f;
+    if (half == 0.f || half * 2.f != w[m]) {
+      int n = 0;
+      for (const bool zero : {true, false})
+        for (int i = 0; i < 4; ++i)
+          if ((weights[i] == 0.f) == zero) {
+            w[n] = weights[i];
+            b[n++] = bones[i];
+          }
+      return;
+    }
+    w[m] = w[k] = half;
+    b[k] = b[m];
+  }
+}
+
 int anim_upload_mesh(anim_ctx *ctx, int32_t type_id, int n_verts, const float *rest_pos, const float *rest_nrm,
                      const int32_t *bones, const float *weights) {
   if (!ctx) return ANIM_EINVAL;
@@ -1476,6 +1509,7 @@ int anim_upload_mesh(anim_ctx *ctx, int32_t type_id, int n_verts, const float *r
   if (!rest_pos || !rest_nrm || !bones || !weights) return fail(ctx, ANIM_EINVAL, "NULL mesh array");
   TypeHost &T = *ctx->types[type_id];
   std::vector<float4> rec((size_t)n_verts * 3);
+  bool zeros = false;
   for (int v = 0; v < n_verts; ++v) {
     for (int k = 0; k < 4; ++k) {
       const int b = bones[4 * v + k];
@@ -1484,25 +1518,10 @@ int anim_upload_mesh(anim_ctx *ctx, int32_t type_id, int n_verts, const float *r
       if (!std::isfinite(w)) return fail(ctx, ANIM_EINVAL, "vertex %d: non-finite weight", v);
     }
     const float *p = rest_pos + 3 * v, *q = rest_nrm + 3 * v;
-    // Zero-weight slots are skipped: each takes half of the weight, and the
-    // bone, of the slot that has the most, so that the kernel need not test
-    // (a branch per slot cost it 5 of 113 us) and no unused bone's pose, be
-    // it non-finite, enters the sum.
     float w[4];
     int32_t b[4];
-    for (int k = 0; k < 4; ++k) {
-      w[k] = weights[4 * v + k];
-      b[k] = bones[4 * v + k];
-    }
-    for (int k = 0; k < 4; ++k) {
-      if (w[k] != 0.f) continue;
-      int m = 0;
-      for (int i = 1; i < 4; ++i)
-        if (std::fabs(w[i]) > std::fabs(w[m])) m = i;
-      w[m] *= 0.5f;
-      w[k] = w[m];
-      b[k] = b[m];
-    }
+    pack_influences(weights + 4 * v, bones + 4 * v, w, b);
+    zeros |= w[0] == 0.f;
     const uint32_t b01 = (uint32_t)b[0] | ((uint32_t)b[1] << 16), b23 = (uint32_t)b[2] | ((uint32_t)b[3] << 16);
     float f01, f23;
     memcpy(&f01, &b01, 4);
@@ -1518,6 +1537,7 @@ int anim_upload_mesh(anim_ctx *ctx, int32_t type_id, int n_verts, const float *r
   CK(cudaMalloc(&T.d_mesh, rec.size() * sizeof(float4)));
   CK(cudaMemcpy(T.d_mesh, rec.data(), rec.size() * sizeof(float4), cudaMemcpyHostToDevice));
   T.n_verts = n_verts;
+  T.mesh_zeros = zeros;
   if (T.d_faces) {  // faces index the mesh they were uploaded for
     cudaFree(T.d_faces);
     T.d_faces = nullptr;

@@ -86,13 +86,16 @@ __device__ __forceinline__ void chain_scan_qt(int n, float4 *P, QT *wtot, int ti
 // goes to sum_k w_k S_{b_k} [p; 1] with normal normalize(sum_k w_k R_{b_k} n)
 // (rigid skin matrices), written as 6 floats at the character's vertex
 // offset.  S is kept in three planes of n rows, character c's from P + c * cs.
-// A thread loads a vertex's record once for the item's characters.
+// A thread loads a vertex's record once for the item's characters.  ZEROS:
+// only the vertices whose first weight is zero, testing their slots; the
+// records of all others have no zero weight (pack_influences).
 // Bound by shared-memory bandwidth: a warp reads 4 bones x 3 rows, 48 wave
 // fronts per 32 vertices, 29 of the about 48 us this pass takes of the 104 us
 // frame (4,097 characters, 1,500 vertices each, 147 MB out; 125 us with the
 // scan on 3x4 matrices, 55 without this pass).  Storing through a staging
 // buffer as consecutive words took 3 us more than these 24-byte rows, the
 // streaming hint 1.5 us less.
+template <bool ZEROS>
 __device__ __forceinline__ void skin_mesh(const ItemBuf &b, const float4 *P, int cs, float *verts, int tid) {
   const int nv = b.T.n_verts, n = b.T.n, C = b.C;
   const float4 *mesh = b.T.mesh;
@@ -100,11 +103,13 @@ __device__ __forceinline__ void skin_mesh(const ItemBuf &b, const float4 *P, int
     const float4 r0 = __ldg(mesh + v), r1 = __ldg(mesh + nv + v), r2 = __ldg(mesh + 2 * nv + v);
     const float w[4] = {r1.z, r1.w, r2.x, r2.y};
     const uint32_t b01 = __float_as_uint(r2.z), b23 = __float_as_uint(r2.w);
+    if (ZEROS && w[0] != 0.f) continue;
     for (int c = 0; c < C; ++c) {
       const float4 *Sc = P + c * cs;
       float px = 0.f, py = 0.f, pz = 0.f, nx = 0.f, ny = 0.f, nz = 0.f;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
+        if (ZEROS && w[k] == 0.f) continue;
         const uint32_t bb = k < 2 ? b01 : b23;
         const float4 *S = Sc + (k & 1 ? bb >> 16 : bb & 0xFFFFu);
         const float4 s0 = S[0], s1 = S[n], s2 = S[2 * n];
@@ -278,7 +283,9 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
     }
     if (MODE == 3) {
       compute_sync();
-      skin_mesh(b, P, cs, a.verts, tid);
+      skin_mesh<false>(b, P, cs, a.verts, tid);
+      // the few meshes with such vertices: their threads write them again
+      if (b.T.mesh_zeros) skin_mesh<true>(b, P, cs, a.verts, tid);
     }
     cur ^= 1;
     handoff_sync();
