@@ -80,6 +80,14 @@ def kernel_source_hash() -> str:
     return h.hexdigest()[:16]
 
 
+def frame_kernels(walked: int, joints: int):
+    """The frame kernel that most of a plan's joints run on, and the launches
+    per frame: the work queue and each of the two frame kernels that has work.
+    walked: the plan's joints on the chain-walk kernel (Context.plan_walk)."""
+    name = "k_walk2 (chain walk in skin space)" if 2 * walked > joints else "k_scan_qt<0> (persistent frame)"
+    return name, 1 + (walked > 0) + (walked < joints)
+
+
 def measured_peaks() -> dict:
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -286,6 +294,7 @@ def run_ours(args) -> dict:
     schedule = ctx.get_schedule(plan)
     joints = plan.total
     n_chars = plan.n_chars
+    frame_kernel, frame_launches = frame_kernels(ctx.plan_walk(plan)[0], plan.total)
     out_bytes = joints * 48
     n_out = max(3, math.ceil(2.5 * L2_BYTES / out_bytes))
     outs = [torch.empty((joints, 12), dtype=torch.float32, device=dev) for _ in range(n_out)]
@@ -375,7 +384,7 @@ def run_ours(args) -> dict:
     tr = NCU_TRAFFIC.get(kernel_source_hash())
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": tr,
-                "kernel": "k_walk2 (chain walk in skin space)" if schedule[3] else "k_scan_qt<0> (persistent frame)",
+                "kernel": frame_kernel,
                 "kernel_ms": round(k_ms, 5), "algorithmic_bytes": alg, "peak_source": peak_src,
                 "nominal_peak": NOMINAL_HBM_GBS, "frac_of_nominal": round(achieved / NOMINAL_HBM_GBS, 4),
                 "touched_bytes": frame_touched_bytes(w)}
@@ -393,9 +402,7 @@ def run_ours(args) -> dict:
                          "schedule": {"seg_len,ctas_per_sm,joints_per_item,walk,adj_ctas": schedule,
                                       "source": "--schedule" if args.schedule else "anim_tune"},
                          "parallelism": f"replicas x{world} (independent character batches)"},
-              # per frame: the work queue, the frame kernel, and with a chain-walk
-              # schedule the segmented kernel beside it (the dragon chain is never walked)
-              "roofline": roofline, "gpu_launches": (3 if schedule[3] else 2) * steps, "clocks": clock}
+              "roofline": roofline, "gpu_launches": frame_launches * steps, "clocks": clock}
 
     # end to end through the C-ABI call with host buffers
     # (anim_evaluate_frame_host): page-locked inputs copied in and the whole
