@@ -377,8 +377,10 @@ ANIM_API int anim_set_schedule(anim_ctx *ctx, anim_plan *plan, const int32_t *in
  * the present schedule: *out_joints receives the number of its joints (0 if
  * all run on the segmented kernel, the plan's total if none do),
  * *out_lanes (nullable) the largest number of lanes a character of these
- * types is walked by (0 without any). */
-ANIM_API int anim_plan_walk(anim_ctx *ctx, const anim_plan *plan, int64_t *out_joints, int32_t *out_lanes);
+ * types is walked by, *out_warps (nullable) which of the kernel's two forms
+ * runs, 1 or 3 warps per work item (both 0 without any). */
+ANIM_API int anim_plan_walk(anim_ctx *ctx, const anim_plan *plan, int64_t *out_joints, int32_t *out_lanes,
+                            int32_t *out_warps);
 
 /* Read and clear the device status word (synchronizes `stream`). */
 ANIM_API int anim_get_status(anim_ctx *ctx, void *stream, int *out_status);

@@ -59,7 +59,7 @@ SIGNATURES = {
     "anim_forward_local_noalloc": (c_int, [c_int, _P, c_int64, _P, _P, _P, _P, _P]),
     "anim_get_schedule": (c_int, [_P, _P, _P]),
     "anim_set_schedule": (c_int, [_P, _P, _P]),
-    "anim_plan_walk": (c_int, [_P, _P, _P, _P]),
+    "anim_plan_walk": (c_int, [_P, _P, _P, _P, _P]),
 }
 
 _lib = None
@@ -340,10 +340,12 @@ class Context:
         return [int(x) for x in out]
 
     def plan_walk(self, plan):
-        """(joints of the plan whose frame runs on the chain-walk kernel, most lanes a character of them takes)"""
-        joints, lanes = ctypes.c_int64(0), ctypes.c_int32(0)
-        self._ck(self.lib.anim_plan_walk(self.h, plan.h, ctypes.byref(joints), ctypes.byref(lanes)))
-        return joints.value, lanes.value
+        """(joints of the plan whose frame runs on the chain-walk kernel, most lanes a character of them takes,
+        warps per work item)"""
+        joints, lanes, warps = ctypes.c_int64(0), ctypes.c_int32(0), ctypes.c_int32(0)
+        self._ck(self.lib.anim_plan_walk(self.h, plan.h, ctypes.byref(joints), ctypes.byref(lanes),
+                                         ctypes.byref(warps)))
+        return joints.value, lanes.value, warps.value
 
     def set_schedule(self, plan, sched):
         """Five values as get_schedule returns; four keep the current adjoint kernel."""

@@ -71,7 +71,7 @@ struct TypeDev {
   int n_faces;
   const float4 *mesh;
   const int32_t *faces;      // [n_faces][3] vertex indices (raster)
-  // Chain-walk frame kernel (k_walk2): a static lane schedule of wk_S steps
+  // Chain-walk frame kernels (k_walk, k_walk2): a static lane schedule of wk_S steps
   // for wk_P lanes per character, staged in chunks of wk_K steps (the table
   // is padded with idle entries to whole chunks); entry [s][slot] names the
   // joint lane `slot` composes at step s (kWInvalid: idle).  wk_mode 1:
@@ -244,10 +244,11 @@ struct AdjointArgs {
 };
 cudaError_t launch_adjoint(int mode, const AdjointArgs &a, const LaunchCfg &cfg, cudaStream_t s);
 
-// Chain-walk frame kernel (three warps per item: two sample and write out,
-// one walks), CTA i running work-queue slot i
+// Chain-walk frame kernels, CTA i running work-queue slot i
 // (at most 32 / wk_P characters of one walk type sharing the key index k0;
-// empty slots exit), composing them lane-parallel along the type's schedule.
+// empty slots exit), composing them lane-parallel along the type's schedule:
+// launch_walk2 with three warps per item (two sample and write out, one
+// walks), launch_walk with one that does it all.
 struct WalkArgs {
   const TypeDev *types;
   const WorkItem *items;
@@ -259,13 +260,16 @@ struct WalkArgs {
   const float *time, *blend_w;
   float *skin;
   // 0: wait for the preceding grid (the work-queue kernel) before reading
-  // the item.  1: the preceding grid is the segmented frame
+  // the item.  1 (launch_walk2 only): the preceding grid is the segmented frame
   // kernel, which lets this launch start only after its own wait for the
   // work queue; the item and the inputs are read from L2 at once, and each
   // CTA waits for that grid at its end, so that the next launch in the
   // stream (the next frame's work queue) still follows both.
   int pred_waited;
 };
+size_t walk_smem_bytes(int chars_per_item, int nbs);
+cudaError_t launch_walk(const WalkArgs &a, size_t smem, cudaStream_t s);
+int walk_blocks_per_sm(size_t smem);  // resident CTAs per SM at this shared-memory size
 size_t walk2_smem_bytes(int chars_per_item, int nbs);
 cudaError_t launch_walk2(const WalkArgs &a, size_t smem, cudaStream_t s);
 int walk2_blocks_per_sm(size_t smem);

@@ -869,6 +869,7 @@ struct anim_plan {
   int n_slots_walk = 0;
   int walk_nbs = 0;
   std::vector<char> on_walk;  // per ctx type id
+  int walk_warps = 3;         // 3: k_walk2, 1: k_walk
   size_t walk_smem = 0;
   // frame with skinning: every type on the segmented CTA kernel (its own
   // range layout when the frame's layout gives some types to the walk kernel)
@@ -1048,9 +1049,16 @@ int choose_C(const anim_ctx *ctx, const TypeHost &T, int kind, int target) {
 // 10.9 us, as 64 items 6.2; 1,000 of them 11.3 and 7.8; the skinned frame of
 // 304 22.1 and 12.5.  From a few waves on the sizes meet (3,000 of 300
 // joints, 9 waves: 34.7 both ways).  `binned`: work items that the frame's
-// queue forms per key index; each non-empty bin of a range then ends with a
-// part-filled item, (C - 1) / 2C of one on average.
+// queue forms per key index.
 constexpr int kBalanceWaves = 3;
+// Work items of C characters that the frame's queue forms of a type: each
+// non-empty key bin of a range ends with a part-filled one, (C - 1) / 2C of it
+// on average.
+double binned_items(int64_t chars, int C, int n_keys, int range) {
+  const double bins =
+      (double)std::min<int64_t>(chars, (chars + range - 1) / range * std::max(1, std::min(n_keys, range)));
+  return (double)chars / C + bins * (C - 1) / (2.0 * C);
+}
 struct BatchType {
   const TypeHost *T;
   int64_t chars;
@@ -1060,13 +1068,7 @@ int item_target(const anim_ctx *ctx, const std::vector<BatchType> &batch, int sl
     double n = 0.0;
     for (const BatchType &t : batch) {
       const int C = std::max(1, choose_C(ctx, *t.T, kind, target));
-      if (binned) {
-        const double bins = (double)std::min<int64_t>(
-            t.chars, (t.chars + kRangeChars - 1) / kRangeChars * std::max(1, std::min(t.T->n_keys, kRangeChars)));
-        n += (double)t.chars / C + bins * (C - 1) / (2.0 * C);
-      } else {
-        n += (double)((t.chars + C - 1) / C);
-      }
+      n += binned ? binned_items(t.chars, C, t.T->n_keys, kRangeChars) : (double)((t.chars + C - 1) / C);
     }
     return n;
   };
@@ -1123,7 +1125,14 @@ std::vector<WorkItem> make_items(const anim_plan *P, const std::vector<int> &Cv)
 //     600 thousand 33.0/32.7, 1.2 million 56.9/42.2;
 //   512-joint bipeds, S about 70: 0.5 million 20.8/27.6, 1.0 million
 //     33.7/32.7, 2.1 million 57.6/47.7.
-// They meet at about 140 to 200 S^2 joints; the line is drawn at 165.
+// They meet at about 140 to 200 S^2 joints; the line is drawn at 165, and up
+// to 13 steps on at most 8 lanes there is none (chains of 10 joints: 12 of
+// them 8.0/7.5, 3,000 10.6/9.2).  One clip halves the walk's sampling: the
+// line lies at 110, and from 20 steps down there is none (67 joints: 12 of
+// them 9.0/8.0, 3,000 18.1/11.7; 120 S^2 joints in chains of 25 12.0/10.4).
+// A step on 16 or 32 lanes, one to a chunk or two, takes longer (12
+// characters of 600 joints, 32 lanes, one clip 10.3/11.1), and beside other
+// types the line stays.
 // All walkable types go if their joints reach that line for the longest
 // schedule among them.  If not, a rare type with a long schedule must not
 // keep a crowd off the walk: the types of the shortest schedules that reach
@@ -1136,29 +1145,67 @@ std::vector<WorkItem> make_items(const anim_plan *P, const std::vector<int> &Cv)
 // trees of 128 joints beside trees of 300, 200 and 25 thousand joints 17.9
 // all segmented, 20.3 apart; 400 and 100 thousand 27.6 and 29.2; but 400 and
 // 25 thousand 23.9 and 23.3, 800 and 100 thousand 37.4 and 35.0.
-constexpr int64_t kWalkJointsPerStep2 = 165;
+int64_t walk_line(int64_t S, bool one_clip, bool small) {
+  return small && S <= (one_clip ? 20 : 13) ? 0 : (one_clip ? 110 : 165) * S * S;
+}
 constexpr int64_t kWalkAloneJoints = 400000, kWalkAloneShare = 8;
 std::vector<char> walk_types(const anim_ctx *ctx, const anim_plan *P, int mode) {
   std::vector<char> on(ctx->types.size(), 0);
   if (mode == kWalkNever) return on;
-  std::vector<std::pair<int64_t, int64_t>> steps;  // (S, joints) of each walkable type
+  struct Walkable {
+    int64_t S, joints;
+    bool one_clip, few_lanes;
+  };
+  std::vector<Walkable> steps;
   for (size_t u = 0; u < P->used.size(); ++u) {
     const TypeHost &T = *ctx->types[P->used[u]];
-    if (T.walk_ready()) steps.push_back({T.ws.S, (int64_t)T.n * (int64_t)P->by_type[u].size()});
+    if (T.walk_ready())
+      steps.push_back({T.ws.S, (int64_t)T.n * (int64_t)P->by_type[u].size(), T.n_clips < 2, T.ws.P <= 8});
   }
-  std::sort(steps.begin(), steps.end());
+  std::sort(steps.begin(), steps.end(), [](const Walkable &a, const Walkable &b) { return a.S < b.S; });
   int64_t most = mode == kWalkAlways ? INT64_MAX : 0, joints = 0;
+  bool one_clip = true, few_lanes = true;
   if (mode == kWalkByBatch)
     for (size_t i = 0; i < steps.size(); ++i) {
-      const int64_t S = steps[i].first;
-      joints += steps[i].second;
-      if (i + 1 < steps.size() && (steps[i + 1].first == S || joints < kWalkAloneJoints ||
+      const int64_t S = steps[i].S;
+      joints += steps[i].joints;
+      one_clip = one_clip && steps[i].one_clip;
+      few_lanes = few_lanes && steps[i].few_lanes;
+      if (i + 1 < steps.size() && (steps[i + 1].S == S || joints < kWalkAloneJoints ||
                                    joints < kWalkAloneShare * (P->total - joints)))
         continue;
-      if (joints >= kWalkJointsPerStep2 * S * S) most = S;
+      if (joints >= walk_line(S, one_clip, few_lanes && joints == P->total)) most = S;
     }
   for (int t : P->used) on[t] = ctx->types[t]->walk_ready() && ctx->types[t]->ws.S <= most;
   return on;
+}
+
+// Warps per item of the chain walk for a plan's walked types: k_walk2's three
+// or k_walk's one.  Two clips cost one warp half as much again per step, and
+// its scattered stores cost long schedules that fill the SM, so that three is
+// the rule.  One warp is the faster
+//   - with one clip and up to 1.5 items per SM, where it has the shorter step:
+//     trees of 67 joints 8.0 us against 9.1, chains of 10 6.1 against 7.1 (at
+//     2.7 and 6 items per SM it turns: 14.8 against 11.7, 13.4 and 11.8);
+//   - where the item slots do not fit the three-warp kernel's 8 resident CTAs
+//     per SM, so that it starts a second wave: 12.2 slots per SM of 67 joints
+//     24.6 against 28.9, 20.4 of them 35.2 against 40.5, 10.3 of 500 (32 lanes)
+//     22.8 against 38.0, 15.9 of a mix of 16 to 200 43.1 against 48.1; on more
+//     than two lanes up to 32 steps (S 38: 52.2 against 47.3; S 70: 59.2
+//     against 46.0).
+// Over 260 random batches of 150 thousand to 2.4 million joints this choice
+// costs 1.5 % over the better one of each, always three warps 7.0 %, one 10.8.
+int walk_warps(const anim_ctx *ctx, const anim_plan *P, int n_slots) {
+  double items = 0.0;
+  bool one_clip = true, shorter = true;
+  for (size_t u = 0; u < P->used.size(); ++u) {
+    if (!P->on_walk[P->used[u]]) continue;
+    const TypeHost &T = *ctx->types[P->used[u]];
+    items += binned_items((int64_t)P->by_type[u].size(), 32 / T.ws.P, T.n_keys, kRangeCharsMax);
+    one_clip = one_clip && T.n_clips < 2;
+    shorter = shorter && (T.ws.S <= 32 || T.ws.P <= 2);
+  }
+  return (one_clip && items <= 1.5 * ctx->sm_count) || (shorter && n_slots > 8.5 * ctx->sm_count) ? 1 : 3;
 }
 
 // (Re)build the schedule-dependent parts of a plan: characters per item,
@@ -1255,10 +1302,15 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
     }
     if (pass == 0) P->n_slots_walk = slots;
   }
+  // a range of the host-buffer frame takes its whole plan's kernel here too
+  P->walk_warps = P->whole ? P->whole->walk_warps : walk_warps(ctx, P, P->n_slots_walk);
   P->walk_smem = 0;
   if (P->n_slots_walk > 0)
-    P->walk_smem = walk2_spread_smem(walk2_smem_bytes(wcmax, P->walk_nbs), P->n_slots_walk, ctx->sm_count);
-  if (P->n_slots_walk > 0 && walk2_blocks_per_sm(P->walk_smem) < 1)
+    P->walk_smem = P->walk_warps == 1
+                       ? walk_smem_bytes(wcmax, P->walk_nbs)
+                       : walk2_spread_smem(walk2_smem_bytes(wcmax, P->walk_nbs), P->n_slots_walk, ctx->sm_count);
+  if (P->n_slots_walk > 0 &&
+      (P->walk_warps == 1 ? walk_blocks_per_sm(P->walk_smem) : walk2_blocks_per_sm(P->walk_smem)) < 1)
     return fail(ctx, ANIM_EUNSUPPORTED, "chain-walk kernel: no resident CTA at %zu bytes of shared memory",
                 P->walk_smem);
   P->n_ranges = (int)ranges.size();
@@ -1765,7 +1817,8 @@ int anim_frame_run_queue(anim_ctx *ctx, const anim_plan *plan, const float *d_ti
   // after it), and the next launch in the stream keeps a single kernel
   // predecessor -- a fork onto the side stream and back ends that chain and
   // costs the next frame its early start.
-  const bool chain = has_walk && has_cta && plan->n_slots - plan->n_slots_walk <= kChainSlots;
+  const bool chain =
+      has_walk && has_cta && plan->walk_warps == 3 && plan->n_slots - plan->n_slots_walk <= kChainSlots;
   if (has_walk && has_cta && !chain) {
     // the two kernels run side by side: fork onto the context's side stream
     if (!ctx->side) {
@@ -1812,7 +1865,7 @@ int anim_frame_run_queue(anim_ctx *ctx, const anim_plan *plan, const float *d_ti
     w.blend_w = d_blend_w;
     w.skin = d_skin;
     w.pred_waited = chain ? 1 : 0;
-    CK(launch_walk2(w, plan->walk_smem, st));
+    CK(plan->walk_warps == 1 ? launch_walk(w, plan->walk_smem, st) : launch_walk2(w, plan->walk_smem, st));
   }
   if (has_walk && has_cta && !chain) {
     CK(cudaEventRecord(ctx->ev_join, ctx->side));
@@ -2597,7 +2650,8 @@ int anim_get_schedule(anim_ctx *ctx, const anim_plan *plan, int32_t *out5) {
   return ANIM_OK;
 }
 
-int anim_plan_walk(anim_ctx *ctx, const anim_plan *plan, int64_t *out_joints, int32_t *out_lanes) {
+int anim_plan_walk(anim_ctx *ctx, const anim_plan *plan, int64_t *out_joints, int32_t *out_lanes,
+                   int32_t *out_warps) {
   int rc = check_plan(ctx, plan);
   if (rc) return rc;
   if (!out_joints) return fail(ctx, ANIM_EINVAL, "out_joints is NULL");
@@ -2611,6 +2665,7 @@ int anim_plan_walk(anim_ctx *ctx, const anim_plan *plan, int64_t *out_joints, in
   }
   *out_joints = joints;
   if (out_lanes) *out_lanes = lanes;
+  if (out_warps) *out_warps = joints ? plan->walk_warps : 0;
   return ANIM_OK;
 }
 

@@ -1,9 +1,9 @@
-"""The chain-walk kernel on batches of every size: a schedule whose fourth
-value is 1 runs every walkable type on it, and anim_plan_walk says so.  Frames
-back to back and in a graph, key counts on both sides of the work queue's 32,
-inverse binds from every source, every lane count from 1 to 32 (chunks of 4, 2
-and 1 steps), forests and joints not numbered depth first, against the oracle
-to the frame tests' tolerance."""
+"""The chain-walk kernels on batches of every size: a schedule whose fourth
+value is 1 runs every walkable type on the walk, with three warps per item or,
+with one clip and few items or past 8.5 item slots per SM, with one; anim_plan_walk says which.  Frames back to back and in a graph, key counts
+on both sides of the work queue's 32, inverse binds from every source, every
+lane count from 1 to 32 (chunks of 4, 2 and 1 steps), forests and joints not
+numbered depth first, against the oracle to the frame tests' tolerance."""
 import numpy as np
 import pytest
 
@@ -24,8 +24,10 @@ def _comb(chains, length):
     return np.array(par, np.int32)
 
 
-def _workload(parents, chars, rng):
+def _workload(parents, chars, rng, clips=2):
     types = [synth.make_type(p, rng, with_clips=True) for p in parents]
+    for t in types:
+        t["keys"] = t["keys"][:clips]
     return {"types": types, "char_type": (np.arange(chars) % len(types)).astype(np.int32),
             "time": rng.uniform(-1, 2, chars).astype(np.float32), "weight": rng.uniform(0, 1, chars).astype(np.float32)}
 
@@ -42,25 +44,42 @@ def _joints(w, types):
     (synth.chain(6), 1), (synth.chain(160), 1), (_comb(2, 12), 2), (_comb(4, 20), 4), (_comb(8, 30), 8),
     (_comb(16, 20), 16), (_comb(32, 10), 32), (np.array([-1] + [0] * 599, np.int32), 32),
     (np.array([-1] + [0] * 63 + list(range(1, 64)), np.int32), 32), (np.array([-1, 0, -1, 2, 2, -1], np.int32), 2)])
-def test_lane_counts(parents, lanes):
-    rng = np.random.default_rng(len(parents))
+@pytest.mark.parametrize("clips", [1, 2])
+def test_lane_counts(parents, lanes, clips):
+    rng = np.random.default_rng(len(parents) + clips)
     for chars in (1, 33, 130):
-        w = _workload([parents], chars, rng)
+        w = _workload([parents], chars, rng, clips)
         ctx, plan = _gpu.setup(w)
         ctx.set_schedule(plan, WALK)
-        assert ctx.plan_walk(plan) == (plan.total, lanes)
+        assert ctx.plan_walk(plan) == (plan.total, lanes, 1 if clips == 1 else 3)
         out = ctx.evaluate_frame(plan, *_inputs(w))
         _gpu.assert_skin_close(out.cpu().numpy(), oracle.frame(w), w)
         ctx.set_schedule(plan, [16, 2, 2048, 0, 0])
-        assert ctx.plan_walk(plan) == (0, 0)
+        assert ctx.plan_walk(plan) == (0, 0, 0)
+
+
+@pytest.mark.parametrize("parents,lanes,chars,warps", [
+    (_comb(32, 10), 32, 1100, 3), (_comb(32, 10), 32, 1400, 1), (_comb(32, 10), 32, 2700, 1),
+    (_comb(16, 20), 16, 2300, 3), (_comb(16, 20), 16, 3000, 1), (_comb(4, 4), 4, 8000, 3), (_comb(4, 4), 4, 12000, 1)])
+def test_warps_by_items(parents, lanes, chars, warps):
+    """Two clips: one warp per item past 8.5 item slots (of 152 SMs) per SM."""
+    rng = np.random.default_rng(chars)
+    w = _workload([parents], chars, rng)
+    ctx, plan = _gpu.setup(w)
+    ctx.set_schedule(plan, WALK)
+    assert ctx.plan_walk(plan) == (plan.total, lanes, warps)
+    out = ctx.evaluate_frame(plan, *_inputs(w))
+    _gpu.assert_skin_close(out.cpu().numpy(), oracle.frame(w), w)
+    assert ctx.status() == 0
 
 
 @pytest.mark.parametrize("dragons", [0, 1, 40])  # none, chained on the stream, side by side
-def test_frames_in_a_row_and_in_a_graph(dragons):
+@pytest.mark.parametrize("clips", [1, 2])
+def test_frames_in_a_row_and_in_a_graph(dragons, clips):
     import torch
-    rng = np.random.default_rng(dragons)
+    rng = np.random.default_rng(dragons * 2 + clips)
     tree = synth.relabel_random_topological(synth.random_tree(67, 14, rng, spine=14), rng)[0]
-    w = _workload([tree, synth.chain(40)], 500, rng)
+    w = _workload([tree, synth.chain(40)], 500, rng, clips)
     w["types"].append(synth.make_type(synth.chain(600), rng, with_clips=True))
     w["char_type"][:dragons] = 2
     frames = [dict(w, time=rng.uniform(0, 1, 500).astype(np.float32), weight=rng.uniform(0, 1, 500).astype(np.float32))
@@ -68,7 +87,7 @@ def test_frames_in_a_row_and_in_a_graph(dragons):
     ref = [oracle.frame(f) for f in frames]
     ctx, plan = _gpu.setup(w)
     ctx.set_schedule(plan, WALK)
-    assert ctx.plan_walk(plan)[0] == _joints(w, (0, 1))
+    assert ctx.plan_walk(plan)[::2] == (_joints(w, (0, 1)), 1 if clips == 1 else 3)
     ins = [_inputs(f) for f in frames]
     outs = [torch.zeros((plan.total, 12), device="cuda") for _ in frames]
     torch.cuda.synchronize()
@@ -97,9 +116,10 @@ def test_frames_in_a_row_and_in_a_graph(dragons):
 
 
 @pytest.mark.parametrize("keys", [2, 3, 32, 33, 40])
-def test_key_counts(keys):
-    rng = np.random.default_rng(keys)
-    w = _workload([synth.random_tree(48, 9, rng, spine=9), synth.chain(64)], 400, rng)
+@pytest.mark.parametrize("clips", [1, 2])
+def test_key_counts(keys, clips):
+    rng = np.random.default_rng(keys + 100 * clips)
+    w = _workload([synth.random_tree(48, 9, rng, spine=9), synth.chain(64)], 400, rng, clips)
     for t in w["types"]:
         k = t["keys"]
         t["keys"] = np.ascontiguousarray(np.concatenate([k] * -(-keys // k.shape[1]), axis=1)[:, :keys])
