@@ -75,6 +75,16 @@ __device__ __forceinline__ Key ldg_key(const float4 *p) {
   return k;
 }
 
+// The same, issued where it stands in the code, ahead of work that does not
+// need it.
+__device__ __forceinline__ Key ldg_key_now(const float4 *p) {
+  Key k;
+  asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(k.q.x), "=f"(k.q.y), "=f"(k.q.z), "=f"(k.q.w), "=f"(k.t.x), "=f"(k.t.y), "=f"(k.t.z), "=f"(k.t.w)
+      : "l"(__cvta_generic_to_global(p)));
+  return k;
+}
+
 // a + f (b - a) of the first three components.
 __device__ __forceinline__ float4 lerp_t(const float4 a, const float4 b, const float f) {
   return make_float4(fmaf(f, b.x - a.x, a.x), fmaf(f, b.y - a.y, a.y), fmaf(f, b.z - a.z, a.z), 0.f);

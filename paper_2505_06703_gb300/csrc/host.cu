@@ -1986,6 +1986,14 @@ int anim_evaluate_frame_host(anim_ctx *ctx, anim_plan *plan, const float *h_time
   return ANIM_OK;
 }
 
+// CTAs of a layered or skinned frame of n_items item slots: one per slot up to
+// the resident ones, but one per SM at least (90 slots of 60 bipeds, layered:
+// 14.8 us with 90 CTAs, 13.4 with 152; 6 of 3 characters of 10 joints 9.1 and
+// 8.6; three per SM for 90 slots 14.9 and 18.9).
+static int frame_ctas(const anim_ctx *ctx, int n_items) {
+  return std::min(ctx->sm_count * ctx->ctas_per_sm, std::max(ctx->sm_count, n_items));
+}
+
 int anim_evaluate_frame_skinned(anim_ctx *ctx, const anim_plan *plan, const float *d_time, const float *d_blend_w,
                                 float *d_skin, float *d_verts, void *stream) {
   int rc = frame_checks(ctx, plan, d_time);
@@ -2021,7 +2029,7 @@ int anim_evaluate_frame_skinned(anim_ctx *ctx, const anim_plan *plan, const floa
   a.verts = d_verts;
   a.vert_off = plan->d_vert_off;
   LaunchCfg cfg = plan->cfg_scan;
-  cfg.ctas = std::max(1, std::min(ctx->sm_count * ctx->ctas_per_sm, a.n_items));
+  cfg.ctas = frame_ctas(ctx, a.n_items);
   cfg.smem = plan->smem_skin;
   CK(launch_scan_qt(3, a, cfg, (cudaStream_t)stream));
   return ANIM_OK;
@@ -2061,7 +2069,10 @@ int anim_evaluate_frame_layers(anim_ctx *ctx, const anim_plan *plan, const float
   a.layer_w = d_weights;
   a.add_w = d_add_w;
   LaunchCfg cfg = plan->cfg_scan;
-  cfg.ctas = std::max(1, std::min(ctx->sm_count * ctx->ctas_per_sm, a.n_items));
+  cfg.ctas = frame_ctas(ctx, a.n_items);
+  // items few enough for two CTAs per SM: the build that samples one character
+  // per thread with the next layer's records on the way
+  if (a.n_items <= 2 * ctx->sm_count) cfg.min_blocks = 2;
   cfg.smem = plan->smem_layers;
   CK(launch_scan_qt(2, a, cfg, (cudaStream_t)stream));
   return ANIM_OK;

@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
       const int W = n * b.cgroups, cpt = b.cpt;
       for (int idx = tid; idx < W; idx += kComputeThreads) {
         const int grp = (int)b.divN.div(idx), j = idx - grp * n;
-        sample_layers(b, j, grp * cpt, min(C, (grp + 1) * cpt), P, cs);
+        sample_layers<MINB == 2>(b, j, grp * cpt, min(C, (grp + 1) * cpt), P, cs);
       }
     } else {
       const int nk = b.T.n_keys, k0 = b.k0, k1 = (k0 + 1 == nk) ? 0 : k0 + 1;

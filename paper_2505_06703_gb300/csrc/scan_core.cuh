@@ -486,10 +486,50 @@ __device__ __forceinline__ ItemLayout item_layout_qt(float4 *sm, int C, int n, i
 // The layered frame of 4,097 bipeds, 4 clips and a layer, a third of the
 // weights 0: 117.2 us with every clip sampled per joint and character and the
 // shares divided out there, 87.9 as it is.
+// ONE: a thread with one character instead keeps its pose in registers and
+// has the next layer's records on the way, used or not, while it samples
+// one.  Small batches' items hold one character and are a chain of latencies:
+// 4 clips and a layer, 3 characters of 10 joints 8.8 us with every clip
+// sampled, 10.1 by the loops over characters, 8.6 so; 60 of 700 joints 32.7,
+// 22.2, 17.5 (both with the CTAs of anim_evaluate_frame_layers).  Its
+// registers cost the 3-CTA build 1.5 of 86.7 us on the large frame.
+template <bool ONE>
 __device__ __forceinline__ void sample_layers(const ItemBuf &b, int j, int c0, int c1, float4 *P, int cs) {
   const int n = b.T.n, nk = b.T.n_keys, k0 = b.k0, k1 = (k0 + 1 == nk) ? 0 : k0 + 1, nc = b.T.n_clips;
   const size_t clip = (size_t)nk * n * 2;
   const float4 *A0 = b.T.keys + ((size_t)k0 * n + j) * 2, *A1 = b.T.keys + ((size_t)k1 * n + j) * 2;
+  if (ONE && c1 - c0 == 1) {
+    const float4 *add = b.T.add_keys;
+    const float al = b.alpha[c0];
+    Key n0 = ldg_key_now(A0), n1 = ldg_key_now(A1);
+    QT x;
+    for (int i = 0; i <= nc; ++i) {
+      const Key a0 = n0, a1 = n1;
+      const float f = i == 0 ? 1.f : i < nc ? b.lf[c0][i - 1] : add ? b.law[c0] : 0.f;
+      if (i + 1 < nc) {
+        A0 += clip;
+        A1 += clip;
+        n0 = ldg_key_now(A0);
+        n1 = ldg_key_now(A1);
+      } else if (i + 1 == nc && add) {
+        n0 = ldg_key_now(add + ((size_t)k0 * n + j) * 2);
+        n1 = ldg_key_now(add + ((size_t)k1 * n + j) * 2);
+      }
+      if (f == 0.f) continue;
+      const float4 q = slerp_pre(a0.q, a1.q, a0.t.w, al), t = lerp_t(a0.t, a1.t, al);
+      if (i == 0) {
+        x = QT{q, t};
+      } else if (i < nc) {
+        x.q = slerp_unit(x.q, q, f);
+        x.t = lerp_t(x.t, t, f);
+      } else {
+        x.q = qmul(x.q, slerp_unit(make_float4(0.f, 0.f, 0.f, 1.f), q, f));
+        x.t = make_float4(fmaf(f, t.x, x.t.x), fmaf(f, t.y, x.t.y), fmaf(f, t.z, x.t.z), 0.f);
+      }
+    }
+    sts_qt(P + c0 * cs, j, n, x);
+    return;
+  }
   {
     const Key a0 = ldg_key(A0), a1 = ldg_key(A1);
     for (int c = c0; c < c1; ++c) {
