@@ -1049,7 +1049,15 @@ int choose_C(const anim_ctx *ctx, const TypeHost &T, int kind, int target) {
 // 10.9 us, as 64 items 6.2; 1,000 of them 11.3 and 7.8; the skinned frame of
 // 304 22.1 and 12.5.  From a few waves on the sizes meet (3,000 of 300
 // joints, 9 waves: 34.7 both ways).  `binned`: work items that the frame's
-// queue forms per key index.
+// queue forms per key index.  Items of a few joints leave most of a CTA idle
+// and gain nothing from being spread, so that binned items and the one-item
+// adjoint's stop at 64 joints: the layered frame of 300 chains of 10 joints 9.9
+// us with items up to the schedule's size, 11.0 with one character each, 9.9
+// so; the adjoint of 1,000 chains of 4 4.3, 5.0, 3.3.  Skinned items go on
+// shrinking, their vertices fill the CTA (300 chains of 4 joints, 300 vertices
+// each: 10.3 against 13.1 us), and the forward's (1,000 chains of 10 joints
+// 5.8 against 6.2).
+constexpr int kSmallItem = 64;
 constexpr int kBalanceWaves = 3;
 // Work items of C characters that the frame's queue forms of a type: each
 // non-empty key bin of a range ends with a part-filled one, (C - 1) / 2C of it
@@ -1072,7 +1080,9 @@ int item_target(const anim_ctx *ctx, const std::vector<BatchType> &batch, int sl
     }
     return n;
   };
-  int lo = 1, hi = ctx->joints_per_item;
+  int hi = ctx->joints_per_item;
+  const bool floor = (kind == 2 && binned) || (kind == 1 && ctx->adj_ctas > 0);
+  int lo = floor ? std::min(kSmallItem, hi) : 1;
   const double waves = std::ceil(items(hi) / slots);
   if (waves > kBalanceWaves) return hi;
   while (lo < hi) {  // items() falls as the target grows
