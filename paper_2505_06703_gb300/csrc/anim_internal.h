@@ -36,14 +36,13 @@ struct TypeDev {
   // joints met on the way to its root: its own seg_link, that of the segment
   // this lies in, and so on.  hang [n_hang]: the segments with a link, x =
   // segment | seg_link << 16, y = the second link or ~0.  Then, for r = 1, 2,
-  // ..., the jump_n[r - 1] segments with more than 2^r links, the lists one after
-  // the other in jump, each in index order (mostly consecutive slots, so few
-  // bank conflicts):
-  // segment | the segment 2^r links up << 12 | (that one's value lies in the
-  // odd buffer after r - 1 jumps) << 24.
+  // ..., the jump_n[r - 1] segments with more than 2^r links, the lists one
+  // after the other in jump [jump_total], each in index order (mostly
+  // consecutive slots, so few bank conflicts): segment | the segment 2^r links
+  // up << 12 | (that one's value lies in the odd buffer after r - 1 jumps) << 24.
   const uint2 *hang;
   const uint32_t *jump;
-  int n_hang, n_jumps;
+  int n_hang, n_jumps, jump_total;
   uint16_t jump_n[kMaxJumps];
   const float4 *inv_bind;    // [n][3] rows of B_i
   const float4 *keys;        // [n_clips][n_keys][n][2]: (qx qy qz qw), (tx ty tz theta); theta's sign

@@ -561,6 +561,7 @@ struct TypeHost {
     dev.jump = (const uint32_t *)(base + o_jump);
     dev.n_hang = (int)seg.hang.size();
     dev.n_jumps = (int)seg.jump_n.size();
+    dev.jump_total = (int)seg.jump.size();
     std::copy(seg.jump_n.begin(), seg.jump_n.end(), dev.jump_n);
     dev.sub16 = (const int16_t *)(base + o_s16);
     dev.par16 = (const int16_t *)(base + o_p16);

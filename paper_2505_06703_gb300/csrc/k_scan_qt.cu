@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(kCtaThreads, MINB) k_scan_qt(const ScanArgs a)
 
     // ---- pass 1a: local poses (q, t) from the clips or the caller's rows;
     // tables staged alongside
+    if (MINB == 2) pass2_touch(b, tid);
     stage_tables(b, Lt, tid);
     if (MODE == 1) {
       // character-major: consecutive lanes read consecutive rows
