@@ -252,7 +252,6 @@ struct WalkArgs {
   const TypeDev *types;
   const WorkItem *items;
   int n_items;                 // slots (the grid)
-  int nbs_max;                 // branch-point slot capacity per character
   const int32_t *item_chars;
   const int64_t *row_off;
   int *status;
@@ -266,10 +265,11 @@ struct WalkArgs {
   // stream (the next frame's work queue) still follows both.
   int pred_waited;
 };
-size_t walk_smem_bytes(int chars_per_item, int nbs);
+// branch_slots: the most branch-point slots an item's characters take together.
+size_t walk_smem_bytes(int branch_slots);
 cudaError_t launch_walk(const WalkArgs &a, size_t smem, cudaStream_t s);
 int walk_blocks_per_sm(size_t smem);  // resident CTAs per SM at this shared-memory size
-size_t walk2_smem_bytes(int chars_per_item, int nbs);
+size_t walk2_smem_bytes(int branch_slots);
 cudaError_t launch_walk2(const WalkArgs &a, size_t smem, cudaStream_t s);
 int walk2_blocks_per_sm(size_t smem);
 // Shared memory per CTA of the warp-specialized walk, padded up from `smem`

@@ -868,7 +868,6 @@ struct anim_plan {
   // (queue counters d_queue[0..1]), the rest to the segmented CTA kernel
   // (d_queue[2..3])
   int n_slots_walk = 0;
-  int walk_nbs = 0;
   std::vector<char> on_walk;  // per ctx type id
   int walk_warps = 3;         // 3: k_walk2, 1: k_walk
   size_t walk_smem = 0;
@@ -1276,9 +1275,8 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   // plain frame: walkable types (chain-walk kernel, 32 / P characters per
   // item) take the first item regions, the others ((q, t) items) follow
   std::vector<int32_t> cap(P->C_frame);
-  int wcmax = 0;
+  int branch_slots = 0;  // of a walk item, its characters' together
   size_t smem_f = 0;
-  P->walk_nbs = 0;
   for (int t : P->used) {
     const TypeHost &T = *ctx->types[t];
     if (!P->on_walk[t]) {
@@ -1286,8 +1284,7 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
       continue;
     }
     cap[t] = 32 / T.ws.P;
-    wcmax = std::max(wcmax, cap[t]);
-    P->walk_nbs = std::max(P->walk_nbs, T.ws.nbs);
+    branch_slots = std::max(branch_slots, cap[t] * T.ws.nbs);
   }
   CK(upload_vec(&P->d_cap, cap));
   // frame work queue: ranges of <= kRangeChars characters of one type, each
@@ -1318,8 +1315,8 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
   P->walk_smem = 0;
   if (P->n_slots_walk > 0)
     P->walk_smem = P->walk_warps == 1
-                       ? walk_smem_bytes(wcmax, P->walk_nbs)
-                       : walk2_spread_smem(walk2_smem_bytes(wcmax, P->walk_nbs), P->n_slots_walk, ctx->sm_count);
+                       ? walk_smem_bytes(branch_slots)
+                       : walk2_spread_smem(walk2_smem_bytes(branch_slots), P->n_slots_walk, ctx->sm_count);
   if (P->n_slots_walk > 0 &&
       (P->walk_warps == 1 ? walk_blocks_per_sm(P->walk_smem) : walk2_blocks_per_sm(P->walk_smem)) < 1)
     return fail(ctx, ANIM_EUNSUPPORTED, "chain-walk kernel: no resident CTA at %zu bytes of shared memory",
@@ -1868,7 +1865,6 @@ int anim_frame_run_queue(anim_ctx *ctx, const anim_plan *plan, const float *d_ti
     w.types = ctx->d_types;
     w.items = plan->d_items_frame;
     w.n_items = plan->n_slots_walk;
-    w.nbs_max = plan->walk_nbs;
     w.item_chars = plan->d_sorted;
     w.row_off = plan->d_row_off;
     w.status = ctx->d_status;

@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(32, 12) k_walk(const WalkArgs a) {
   x.u = T.wk_u;
   x.tab = T.wk_tab;
   unsigned char *stage = wsm;
-  x.bslots = reinterpret_cast<float4 *>(wsm + kStages * kChunkBytes) + (size_t)x.c * a.nbs_max * 3;
+  x.bslots = reinterpret_cast<float4 *>(wsm + kStages * kChunkBytes) + (size_t)x.c * T.wk_nbs * 3;
   uint32_t parity = 0, inflight = 0;
   bool ok;
   switch (T.wk_K) {
@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(32, 12) k_walk(const WalkArgs a) {
 
 }  // namespace
 
-size_t walk_smem_bytes(int chars_per_item, int nbs) {
-  return (size_t)kStages * kChunkBytes + 48ull * (size_t)chars_per_item * (size_t)nbs;
+size_t walk_smem_bytes(int branch_slots) {
+  return (size_t)kStages * kChunkBytes + 48ull * (size_t)branch_slots;
 }
 
 int walk_blocks_per_sm(size_t smem) {

@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(kW2Threads, 8) k_walk2(const WalkArgs a) {
       else w2_issue<4>(it, q, sm + q * kRecBuf, &B.rec_full[q]);
     }
   }
-  float4 *bslots = reinterpret_cast<float4 *>(sm + kSlotOff) + (size_t)c * a.nbs_max * 3;
+  float4 *bslots = reinterpret_cast<float4 *>(sm + kSlotOff) + (size_t)c * T.wk_nbs * 3;
   bool ok;
   if (warp == 0) {
     ok = it.K == 1   ? w2_walker<1>(it, sm, B, bslots)
@@ -397,8 +397,8 @@ __global__ void __launch_bounds__(kW2Threads, 8) k_walk2(const WalkArgs a) {
 
 }  // namespace
 
-size_t walk2_smem_bytes(int chars_per_item, int nbs) {
-  return (size_t)kSlotOff + 48ull * (size_t)chars_per_item * (size_t)nbs;
+size_t walk2_smem_bytes(int branch_slots) {
+  return (size_t)kSlotOff + 48ull * (size_t)branch_slots;
 }
 
 namespace {

@@ -73,6 +73,20 @@ def test_warps_by_items(parents, lanes, chars, warps):
     assert ctx.status() == 0
 
 
+def test_many_characters_beside_many_branch_points():
+    """A type of 32 characters per item beside one of some 170 branch-point slots per character: each item takes the
+    slots its own type needs (the largest of both at once would not fit a CTA)."""
+    rng = np.random.default_rng(3)
+    tree = synth.relabel_dfs(synth.random_tree(1000, 40, rng, spine=40), rng)[0]
+    w = _workload([synth.chain(6), tree, _comb(8, 30)], 90, rng)
+    ctx, plan = _gpu.setup(w)
+    ctx.set_schedule(plan, WALK)
+    assert ctx.plan_walk(plan)[0] == plan.total
+    out = ctx.evaluate_frame(plan, *_inputs(w))
+    _gpu.assert_skin_close(out.cpu().numpy(), oracle.frame(w), w)
+    assert ctx.status() == 0
+
+
 @pytest.mark.parametrize("dragons", [0, 1, 40])  # none, chained on the stream, side by side
 @pytest.mark.parametrize("clips", [1, 2])
 def test_frames_in_a_row_and_in_a_graph(dragons, clips):
