@@ -1142,7 +1142,11 @@ std::vector<WorkItem> make_items(const anim_plan *P, const std::vector<int> &Cv)
 // them 9.0/8.0, 3,000 18.1/11.7; 120 S^2 joints in chains of 25 12.0/10.4).
 // A step on 16 or 32 lanes, one to a chunk or two, takes longer (12
 // characters of 600 joints, 32 lanes, one clip 10.3/11.1), and beside other
-// types the line stays.
+// types the line stays.  With 64 keys and more a segmented item, the
+// characters of one key of 256, holds few; for the one or two lanes of long
+// chains the walk then pays from 95 S^2 joints on, with one clip from 60 (90
+// keys: 100 S^2 joints in chains of 60 32.1/28.4 us, with one clip 29.6/23.9;
+// 60 S^2 in chains of 25, one clip, 12.0/10.9).
 // All walkable types go if their joints reach that line for the longest
 // schedule among them.  If not, a rare type with a long schedule must not
 // keep a crowd off the walk: the types of the shortest schedules that reach
@@ -1155,8 +1159,9 @@ std::vector<WorkItem> make_items(const anim_plan *P, const std::vector<int> &Cv)
 // trees of 128 joints beside trees of 300, 200 and 25 thousand joints 17.9
 // all segmented, 20.3 apart; 400 and 100 thousand 27.6 and 29.2; but 400 and
 // 25 thousand 23.9 and 23.3, 800 and 100 thousand 37.4 and 35.0.
-int64_t walk_line(int64_t S, bool one_clip, bool small) {
-  return small && S <= (one_clip ? 20 : 13) ? 0 : (one_clip ? 110 : 165) * S * S;
+int64_t walk_line(int64_t S, bool one_clip, bool small, bool few_per_key) {
+  if (small && S <= (one_clip ? 20 : 13)) return 0;
+  return (few_per_key ? (one_clip ? 60 : 95) : one_clip ? 110 : 165) * S * S;
 }
 constexpr int64_t kWalkAloneJoints = 400000, kWalkAloneShare = 8;
 std::vector<char> walk_types(const anim_ctx *ctx, const anim_plan *P, int mode) {
@@ -1164,27 +1169,29 @@ std::vector<char> walk_types(const anim_ctx *ctx, const anim_plan *P, int mode) 
   if (mode == kWalkNever) return on;
   struct Walkable {
     int64_t S, joints;
-    bool one_clip, few_lanes;
+    bool one_clip, few_lanes, few_per_key;
   };
   std::vector<Walkable> steps;
   for (size_t u = 0; u < P->used.size(); ++u) {
     const TypeHost &T = *ctx->types[P->used[u]];
     if (T.walk_ready())
-      steps.push_back({T.ws.S, (int64_t)T.n * (int64_t)P->by_type[u].size(), T.n_clips < 2, T.ws.P <= 8});
+      steps.push_back({T.ws.S, (int64_t)T.n * (int64_t)P->by_type[u].size(), T.n_clips < 2, T.ws.P <= 8,
+                       T.ws.P <= 2 && T.n_keys >= 64});
   }
   std::sort(steps.begin(), steps.end(), [](const Walkable &a, const Walkable &b) { return a.S < b.S; });
   int64_t most = mode == kWalkAlways ? INT64_MAX : 0, joints = 0;
-  bool one_clip = true, few_lanes = true;
+  bool one_clip = true, few_lanes = true, few_per_key = true;
   if (mode == kWalkByBatch)
     for (size_t i = 0; i < steps.size(); ++i) {
       const int64_t S = steps[i].S;
       joints += steps[i].joints;
       one_clip = one_clip && steps[i].one_clip;
       few_lanes = few_lanes && steps[i].few_lanes;
+      few_per_key = few_per_key && steps[i].few_per_key;
       if (i + 1 < steps.size() && (steps[i + 1].S == S || joints < kWalkAloneJoints ||
                                    joints < kWalkAloneShare * (P->total - joints)))
         continue;
-      if (joints >= walk_line(S, one_clip, few_lanes && joints == P->total)) most = S;
+      if (joints >= walk_line(S, one_clip, few_lanes && joints == P->total, few_per_key)) most = S;
     }
   for (int t : P->used) on[t] = ctx->types[t]->walk_ready() && ctx->types[t]->ws.S <= most;
   return on;
@@ -1200,22 +1207,27 @@ std::vector<char> walk_types(const anim_ctx *ctx, const anim_plan *P, int mode) 
 //   - where the item slots do not fit the three-warp kernel's 8 resident CTAs
 //     per SM, so that it starts a second wave: 12.2 slots per SM of 67 joints
 //     24.6 against 28.9, 20.4 of them 35.2 against 40.5, 10.3 of 500 (32 lanes)
-//     22.8 against 38.0, 15.9 of a mix of 16 to 200 43.1 against 48.1; on more
-//     than two lanes up to 32 steps (S 38: 52.2 against 47.3; S 70: 59.2
-//     against 46.0).
+//     22.8 against 38.0, 15.9 of a mix of 16 to 200 43.1 against 48.1.  On
+//     more than two lanes up to 32 steps (12.4 slots, S 38: 52.2 against 47.3;
+//     10.6, S 70: 59.2 against 46.0), while the second wave is nearly empty up
+//     to 50 and on 16 lanes and more (10.1 slots, S 46: 43.2 against 51.5; 10.5
+//     of 700 joints, S 60, 16 lanes: 61.8 against 78.6).
 // Over 260 random batches of 150 thousand to 2.4 million joints this choice
-// costs 1.5 % over the better one of each, always three warps 7.0 %, one 10.8.
+// costs 1.2 % over the better one of each, always three warps 7.0 %, one 10.8.
 int walk_warps(const anim_ctx *ctx, const anim_plan *P, int n_slots) {
   double items = 0.0;
-  bool one_clip = true, shorter = true;
+  bool one_clip = true, brief = true, medium = true;
   for (size_t u = 0; u < P->used.size(); ++u) {
     if (!P->on_walk[P->used[u]]) continue;
     const TypeHost &T = *ctx->types[P->used[u]];
     items += binned_items((int64_t)P->by_type[u].size(), 32 / T.ws.P, T.n_keys, kRangeCharsMax);
     one_clip = one_clip && T.n_clips < 2;
-    shorter = shorter && (T.ws.S <= 32 || T.ws.P <= 2);
+    brief = brief && (T.ws.S <= 32 || T.ws.P <= 2);
+    medium = medium && (T.ws.S <= 50 || T.ws.P <= 2 || T.ws.P >= 16);
   }
-  return (one_clip && items <= 1.5 * ctx->sm_count) || (shorter && n_slots > 8.5 * ctx->sm_count) ? 1 : 3;
+  const double slots = (double)n_slots / ctx->sm_count;
+  const bool one = slots > 8.5 ? brief || (medium && slots <= 11.7) : one_clip && items <= 1.5 * ctx->sm_count;
+  return one ? 1 : 3;
 }
 
 // (Re)build the schedule-dependent parts of a plan: characters per item,
