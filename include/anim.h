@@ -117,8 +117,11 @@ ANIM_API int anim_create_skeletons(anim_ctx *ctx, int n_types, const int32_t *jo
  * 1 <= n_clips <= ANIM_MAX_CLIPS (anim_evaluate_frame blends clip 0 -> clip
  * 1 by the per-character weight; anim_evaluate_frame_layers blends all of
  * them), 2 <= n_keys <= ANIM_MAX_KEYS, keys looping with period n_keys /
- * rate_hz seconds.  Replaces earlier clips of the type (and drops an
- * additive layer whose key count or rate no longer matches).  Synchronous. */
+ * rate_hz seconds.  Rotations of unit length are meant; of others the
+ * chain-walk kernel normalizes each key, the segmented one the slerp of two
+ * as stored, so that what they give depends on the kernel a type runs on.
+ * Replaces earlier clips of the type (and drops an additive layer whose key
+ * count or rate no longer matches).  Synchronous. */
 ANIM_API int anim_upload_clips(anim_ctx *ctx, int32_t type_id, int n_clips, int n_keys, float rate_hz, const float *keys);
 
 /* An additive layer for a type (the paper asks for the clip blending of an
@@ -166,10 +169,11 @@ ANIM_API int anim_plan_vertex_offsets(anim_ctx *ctx, const anim_plan *plan, int6
  * bind.  d_time, d_blend_w: device [n_chars] float; d_skin: device
  * [total][12] float (written).  A small work-queue launch, then the frame
  * kernels: the segmented persistent kernel for the types without a
- * chain-walk schedule and, under a schedule that enables it and in batches
- * large enough for it to be the faster one, the chain-walk kernel for the others -- one after the other on `stream` when the
- * segmented part holds at most 16 work items, otherwise side by side on a
- * second stream of the context that `stream` forks to and joins back. */
+ * chain-walk schedule and the chain-walk kernel for others as the schedule
+ * says (anim_get_schedule; anim_plan_walk tells which ran) -- one after the
+ * other on `stream` when the segmented part holds at most 16 work items and
+ * the walk has three warps per item, otherwise side by side on a second
+ * stream of the context that `stream` forks to and joins back. */
 ANIM_API int anim_evaluate_frame(anim_ctx *ctx, const anim_plan *plan, const float *d_time, const float *d_blend_w,
                         float *d_skin, void *stream);
 
@@ -331,8 +335,8 @@ ANIM_API int anim_ik_step(anim_ctx *ctx, anim_ik *ik, float *d_q, float *d_m, fl
  * pointer-jumping scan, 1, 2 or 3 resident CTAs per SM of the persistent
  * kernels, work items of about 1,024/2,048/4,096 joints, and for the
  * frame whether walkable types (chain schedules of at most 160 steps with
- * most lanes busy) run on the chain-walk kernel beside the segmented kernel
- * -- of
+ * most lanes busy) run on the chain-walk kernel by batch, never or always,
+ * where these differ -- of
  * `which` (0 = fused frame, 1 = forward_local, 2 = loss_backward, 3 = frame
  * with skinning, 4 = frame with layered blending) with CUDA events on scratch
  * inputs it allocates, and keeps the fastest.  The result

@@ -211,9 +211,9 @@ __device__ __forceinline__ void test_pixel(const RasterArgs &a, const WarpTris &
 // Measured (4,097 characters of 1,498 faces, 1920x1080, 40 % of them below
 // the image, all three launches): 422 us with a triangle per lane in 64-bit
 // arithmetic from global vertices, 226 with staged vertices and 32-bit
-// edges, 176 with a row per lane, 112 as it is (83.8 M warp instructions at
-// 75 % issue; the vertices' 147 MB take 22 us).  A 5-CTA build spills: 116;
-// three CTAs per SM: 122.
+// edges, 176 with a row per lane, 109 as it is (82.3 M warp instructions at
+// 76 % issue; the vertices' 147 MB take 22 us).  A 5-CTA build spills: 116
+// against 112; three CTAs per SM: 122.
 // ALL_STAGED: every mesh fits the stage.  Otherwise the characters of the
 // larger ones snap each triangle's corners as they come to it: 1,500 of 4,500
 // vertices and 4,096 faces, 64 columns, take 177 us (686 with a triangle per
