@@ -1057,6 +1057,15 @@ int choose_C(const anim_ctx *ctx, const TypeHost &T, int kind, int target) {
 // shrinking, their vertices fill the CTA (300 chains of 4 joints, 300 vertices
 // each: 10.3 against 13.1 us), and the forward's (1,000 chains of 10 joints
 // 5.8 against 6.2).
+// `by_largest`: nor do items go below half of the largest type's character
+// (that character's item sets the time, and smaller items of the others only
+// crowd its SM), or below the whole of it where it has four times the joints
+// of the average one; the forward and the frames only within one wave.  The
+// five mixed types (32 to 2,048 joints), 300 / 1,100 characters: forward with
+// three CTAs per SM 16.3 / 22.3 us without this, 12.0 / 16.7 with it (12.4 /
+// 16.9 at the schedule's size), layered 34.6 / 44.5, 29.4 / 40.5 (33.0 /
+// 42.8), one-item adjoint of 3,000 138.9, 121.3 (122.7).  Without: skinned
+// items (503 characters 24.4 against 27.1) and IK's (60 12.7 against 13.3).
 constexpr int kSmallItem = 64;
 constexpr int kBalanceWaves = 3;
 // Work items of C characters that the frame's queue forms of a type: each
@@ -1071,7 +1080,8 @@ struct BatchType {
   const TypeHost *T;
   int64_t chars;
 };
-int item_target(const anim_ctx *ctx, const std::vector<BatchType> &batch, int slots, int kind, bool binned) {
+int item_target(const anim_ctx *ctx, const std::vector<BatchType> &batch, int slots, int kind, bool binned,
+                bool by_largest) {
   auto items = [&](int target) {
     double n = 0.0;
     for (const BatchType &t : batch) {
@@ -1085,6 +1095,16 @@ int item_target(const anim_ctx *ctx, const std::vector<BatchType> &batch, int sl
   int lo = floor ? std::min(kSmallItem, hi) : 1;
   const double waves = std::ceil(items(hi) / slots);
   if (waves > kBalanceWaves) return hi;
+  if (by_largest && (kind == 1 || waves <= 1)) {
+    int64_t most = 0, joints = 0, chars = 0;
+    for (const BatchType &t : batch) {
+      most = std::max<int64_t>(most, t.T->n);
+      joints += t.T->n * t.chars;
+      chars += t.chars;
+    }
+    const bool rare = kind != 1 && most * chars >= 4 * joints;
+    lo = (int)std::max<int64_t>(lo, std::min<int64_t>(hi, rare ? most : most / 2));
+  }
   while (lo < hi) {  // items() falls as the target grows
     const int mid = (lo + hi) / 2;
     if (items(mid) <= waves * slots) hi = mid;
@@ -1252,9 +1272,9 @@ int plan_schedule(anim_ctx *ctx, anim_plan *P) {
     if (!P->on_walk[P->used[u]]) seg.push_back({&T, cnt});
   }
   const int ctas = ctx->sm_count * ctx->ctas_per_sm;
-  const int t_fwd = item_target(ctx, all, ctas, 2, false), t_frame = item_target(ctx, seg, ctas, 2, true),
-            t_layers = item_target(ctx, all, ctas, 2, true), t_skin = item_target(ctx, all, ctas, 3, true),
-            t_adj = item_target(ctx, adj, adj_slots(ctx), 1, false);
+  const int t_fwd = item_target(ctx, all, ctas, 2, false, true), t_frame = item_target(ctx, seg, ctas, 2, true, true),
+            t_layers = item_target(ctx, all, ctas, 2, true, true), t_skin = item_target(ctx, all, ctas, 3, true, false),
+            t_adj = item_target(ctx, adj, adj_slots(ctx), 1, false, true);
   for (int t : P->used) {
     const TypeHost &T = *ctx->types[t];
     const int cs = choose_C(ctx, T, 0, 1), ca = choose_C(ctx, *T.adj, 1, t_adj);
@@ -2279,7 +2299,7 @@ int anim_ik_create(anim_ctx *ctx, const anim_plan *plan, int n_eff, const int32_
   std::vector<BatchType> batch;
   for (size_t u = 0; u < plan->used.size(); ++u)
     batch.push_back({K->views[plan->used[u]].get(), (int64_t)plan->by_type[u].size()});
-  const int target = item_target(ctx, batch, adj_slots(ctx), 1, false);
+  const int target = item_target(ctx, batch, adj_slots(ctx), 1, false, false);
   for (int t : plan->used) {
     const TypeHost &V = *K->views[t];
     const int C = choose_C(ctx, V, 1, target);
