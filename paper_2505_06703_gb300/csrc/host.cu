@@ -1060,12 +1060,15 @@ int choose_C(const anim_ctx *ctx, const TypeHost &T, int kind, int target) {
 // `by_largest`: nor do items go below half of the largest type's character
 // (that character's item sets the time, and smaller items of the others only
 // crowd its SM), or below the whole of it where it has four times the joints
-// of the average one; the forward and the frames only within one wave.  The
-// five mixed types (32 to 2,048 joints), 300 / 1,100 characters: forward with
-// three CTAs per SM 16.3 / 22.3 us without this, 12.0 / 16.7 with it (12.4 /
-// 16.9 at the schedule's size), layered 34.6 / 44.5, 29.4 / 40.5 (33.0 /
-// 42.8), one-item adjoint of 3,000 138.9, 121.3 (122.7).  Without: skinned
-// items (503 characters 24.4 against 27.1) and IK's (60 12.7 against 13.3).
+// of the average one; the forward and the frames only within one wave, with
+// three CTAs per SM the forward within two.  The five mixed types (32 to 2,048
+// joints), 300 / 1,100 / 2,344 characters: forward with three CTAs per SM 16.3
+// / 22.3 / 34.2 us without this, 12.0 / 16.7 / 28.7 with it (12.4 / 16.9 /
+// 30.1 at the schedule's size; in two waves of two CTAs per SM, 1,500
+// characters, 22.6 and 25.9); layered 300 / 1,100 34.6 / 44.5, 29.4 / 40.5
+// (33.0 / 42.8); one-item adjoint of 3,000 138.9, 121.3 (122.7).  Without:
+// skinned items (503 characters 24.4 against 27.1) and IK's (60 12.7 against
+// 13.3).
 constexpr int kSmallItem = 64;
 constexpr int kBalanceWaves = 3;
 // Work items of C characters that the frame's queue forms of a type: each
@@ -1095,7 +1098,7 @@ int item_target(const anim_ctx *ctx, const std::vector<BatchType> &batch, int sl
   int lo = floor ? std::min(kSmallItem, hi) : 1;
   const double waves = std::ceil(items(hi) / slots);
   if (waves > kBalanceWaves) return hi;
-  if (by_largest && (kind == 1 || waves <= 1)) {
+  if (by_largest && (kind == 1 || waves <= (!binned && ctx->ctas_per_sm >= 3 ? 2 : 1))) {
     int64_t most = 0, joints = 0, chars = 0;
     for (const BatchType &t : batch) {
       most = std::max<int64_t>(most, t.T->n);
